@@ -631,8 +631,9 @@ int bcq_pack(const bcq_desc *desc, const uint8_t *codes, const uint16_t *alpha_i
         return BCQ_ERR_MISALIGNED;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const View dst = make_view(*desc, packed, alpha_out, z_out);
-    cudaError_t e = launch_pack(codes, dst, st);
-    if (e == cudaSuccess && scales) {
+    const bool in_tiles = interleaved(desc);   // the scales go into the tiles together with the planes
+    cudaError_t e = launch_pack(codes, in_tiles ? alpha_in : nullptr, in_tiles ? z_in : nullptr, dst, st);
+    if (e == cudaSuccess && scales && !in_tiles) {
         bcq_desc canon = *desc;
         canon.layout = BCQ_LAYOUT_CANONICAL;
         e = launch_permute_scales(make_view(canon, nullptr, alpha_in, z_in), dst, st);
