@@ -183,8 +183,8 @@ int bcq_merge_linear(const bcq_desc *desc, const uint8_t *w_int_dev, const uint1
  * the kernels' scratch); w_int [N][K] or NULL; packed / alpha / z exactly as bcq_merge_linear
  * followed by bcq_pack would produce them for desc->layout (alpha and z ignored when the tiles
  * carry the scales).  Asynchronous on `stream`, no allocation.  The paper times no quantiser;
- * this one reads W once for groups of 128 (2 bytes per weight plus the operand written) and
- * twice (range, then encode) for every other group length.
+ * this one reads W once for groups of 128, 64 and 32 (2 bytes per weight plus the operand
+ * written) and twice (range, then encode; the second time from L2) for every other group length.
  */
 int bcq_quantize_rtn(const bcq_desc *desc, const uint16_t *W_dev, int n_bits,
                      const uint8_t *bit_to_plane_host, double s_factor, uint16_t *S_dev,

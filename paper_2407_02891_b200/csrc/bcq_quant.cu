@@ -9,13 +9,18 @@
 //
 // The quantiser is the inverse of the dequantisation S W_int + qbias and uses the fp16 S that is
 // stored.  The integer is defined in fp64: W - qbias is exact there, the quotient is rounded once,
-// so the decision does not depend on evaluation order.  Groups of 128 take one pass over W (a
-// group's 16 chunks sit in 16 lanes); other group lengths take a range pass and an encode pass.
-#include "bcq_internal.cuh"
+// so the decision does not depend on evaluation order.
+//
+// One kernel.  A warp takes one 128-weight segment of eight rows at a time, 32 weights per lane (see bcq_planes.cuh).
+// Groups of 128, 64 and 32 are 4, 2 and 1 of those lanes: range by shuffles, one pass over W.  Other group lengths (and
+// one scale per row) take the range first, eight rows per block, and read the rows a second time from L2.
+//
+// Bound: instruction issue (23 instructions per weight, issue slots 68 % busy), then HBM (2 bytes
+// per weight).  7168 x 7168, q = 3, groups of 128: 201 us with a chunk of 8 weights per thread, byte stores and a 16-lane
+// range reduction; 52 us so (2.4 TB/s).
+#include "bcq_planes.cuh"
 
 namespace bcq {
-
-constexpr int kQuantRows = 16;   // rows a block walks: the block's table set-up is shared by them
 
 struct QuantTable {
     uint8_t code_of_int[256];
@@ -25,110 +30,6 @@ struct QuantTable {
     double s_factor;
 };
 
-// One warp per (row, group): the range of the group's weights, then S and qbias.
-__global__ void __launch_bounds__(256) rtn_range_kernel(const __half *__restrict__ W, int N, int K, int L, QuantTable tab,
-                                                        __half *__restrict__ S, __half *__restrict__ qbias)
-{
-    const int G = K / L;
-    const size_t unit = (size_t(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-    const int lane = threadIdx.x & 31;
-    if (unit >= size_t(N) * G) return;
-    const __half *w = W + (unit / G) * size_t(K) + (unit % G) * size_t(L);
-    float lo = __half2float(w[0]), hi = lo;
-#pragma unroll 4
-    for (int k = 8 * lane; k < L; k += 256) {   // L is a multiple of 32: whole 16-byte pieces
-        const uint4 raw = *reinterpret_cast<const uint4 *>(w + k);
-        const __half2 *h = reinterpret_cast<const __half2 *>(&raw);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const float2 f = __half22float2(h[j]);
-            lo = fminf(lo, fminf(f.x, f.y));
-            hi = fmaxf(hi, fmaxf(f.x, f.y));
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    }
-    if (lane == 0) {
-        if (lo == 0.f) lo = 0.f;   // a zero minimum is stored as +0
-        const double range = double(hi) - double(lo);   // exact
-        S[unit] = __double2half(__ddiv_rn(__dmul_rn(tab.s_factor, range), tab.top));
-        qbias[unit] = __float2half_rn(lo);              // exact: lo is an fp16 value
-    }
-}
-
-// Shared-memory table of a block: entry t = the code of step-1 integer t with code bit i moved to
-// bit 8 i, so that OR-ing (entry << j) over the 8 weights j of a chunk leaves plane i's byte in byte i.
-__device__ __forceinline__ void load_spread_table(const QuantTable &tab, uint32_t *lut)
-{
-    for (int t = threadIdx.x; t < 256; t += blockDim.x) {
-        const uint32_t c = tab.code_of_int[t];
-        lut[t] = (c & 1u) | ((c & 2u) << 7) | ((c & 4u) << 14) | ((c & 8u) << 21);
-    }
-    __syncthreads();
-}
-
-// Integers, codes and plane bytes of one chunk of 8 weights (row n, bytes kb of the planes).
-// The integer is DEFINED by the fp64 quotient (W - qbias)/S, rounded to nearest, ties to even.  An
-// fp32 estimate t of the quotient (three roundings, relative error below 1.8e-7) decides whenever it
-// is further from a rounding boundary than its own error bound; the few weights that are not (and
-// exact ties) take the fp64 division.  Same integers, a fraction of the fp64 work.  Rounding t: adding
-// 1.5 * 2^23 leaves the nearest integer in the low mantissa bits (valid below 2^22; larger t clamp).
-// PACK = false (the search over scale factors wants the integers only): no codes, no plane bytes.
-template <bool PACK>
-__device__ __forceinline__ void encode_chunk(const uint4 raw, __half s_h, __half b_h, const QuantTable &tab,
-                                             const uint32_t *lut, uint8_t *__restrict__ w_int, const View &dst, int n, int kb)
-{
-    const float sf = __half2float(s_h), bf = __half2float(b_h);
-    const float inv_s = sf > 0.f ? __frcp_rn(sf) : 0.f;   // S = 0: every t is 0, every integer 0
-    const float topf = float(tab.top);
-    const int topi = int(tab.top);
-    const float magic = 12582912.f;
-    const uint32_t word[4] = {raw.x, raw.y, raw.z, raw.w};
-    uint32_t spread = 0u, ints_lo = 0u, ints_hi = 0u;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        const __half hw = __ushort_as_half(uint16_t(word[j >> 1] >> (16 * (j & 1))));
-        const float w = __half2float(hw);
-        const float t = __fmul_rn(__fsub_rn(w, bf), inv_s);   // >= 0: qbias is the minimum
-        const float err = fmaf(t, 4e-7f, 1e-6f);
-        int r;
-        if (t - err > topf + 0.5f) {
-            r = topi;
-        } else {
-            const float shifted = __fadd_rn(t, magic);
-            const float nearest = __fsub_rn(shifted, magic);
-            if (fabsf(t - nearest) < 0.5f - err) {
-                r = min(__float_as_int(shifted) - __float_as_int(magic), topi);
-            } else {
-                const double r64 = rint(__ddiv_rn(double(w) - double(bf), double(sf)));   // the subtraction is exact in fp64
-                r = int(fmin(fmax(r64, 0.0), tab.top));
-            }
-        }
-        if (PACK) spread |= lut[r] << j;
-        if (j < 4)
-            ints_lo |= uint32_t(r) << (8 * j);
-        else
-            ints_hi |= uint32_t(r) << (8 * (j - 4));
-    }
-    if (PACK) {
-        unsigned char *out = dst.plane_byte(0, n, kb);
-        const size_t stride = dst.plane_stride();
-        for (int i = 0; i < dst.q; ++i) out[i * stride] = uint8_t(spread >> (8 * i));
-    }
-    if (w_int) *reinterpret_cast<uint2 *>(w_int + size_t(n) * dst.K + size_t(kb) * 8) = make_uint2(ints_lo, ints_hi);
-}
-
-// alpha_j = S m_j and z = S centre + qbias of one (row, group): exact in fp64, rounded once.
-__device__ __forceinline__ void write_scales(__half s_h, __half b_h, const QuantTable &tab, const View &dst, int n, int g)
-{
-    const double s = double(__half2float(s_h)), b = double(__half2float(b_h));
-    for (int j = 0; j < dst.q; ++j) *dst.alpha_elem(j, n, g) = __half_as_ushort(__double2half(s * tab.plane_weight[j]));
-    *dst.z_elem(n, g) = __half_as_ushort(__double2half(s * tab.centre + b));
-}
-
 __device__ __forceinline__ void range_to_scale(float lo, float hi, const QuantTable &tab, __half &s_h, __half &b_h)
 {
     if (lo == 0.f) lo = 0.f;   // a zero minimum is stored as +0
@@ -137,94 +38,270 @@ __device__ __forceinline__ void range_to_scale(float lo, float hi, const QuantTa
     b_h = __float2half_rn(lo);                      // exact: lo is an fp16 value
 }
 
-// Any group length: one thread per (row, chunk), S and qbias from the range kernel.  Block (x, y) covers
-// rows kQuantRows x .. + kQuantRows - 1 and chunks 256 y .. + 255.
-template <bool PACK>
-__global__ void __launch_bounds__(256) rtn_encode_kernel(const __half *__restrict__ W, const __half *__restrict__ S,
-                                                         const __half *__restrict__ qbias, int L, QuantTable tab,
-                                                         uint8_t *__restrict__ w_int, const View dst)
+// alpha_j = S m_j (j < q), z = S centre + qbias (j = q) of one (row, group): exact in fp64, rounded once.
+__device__ __forceinline__ uint16_t fused_scale(__half s_h, __half b_h, const QuantTable &tab, int q, int j)
 {
-    __shared__ uint32_t lut[256];
-    load_spread_table(tab, lut);
-    const int kb = blockIdx.y * 256 + threadIdx.x;
-    if (kb >= dst.K / 8) return;
-    const int G = dst.K / L, g = (kb * 8) / L;
-    for (int n = blockIdx.x * kQuantRows; n < min(dst.N, (blockIdx.x + 1) * kQuantRows); ++n) {
-        const uint4 raw = *reinterpret_cast<const uint4 *>(W + size_t(n) * dst.K + size_t(kb) * 8);
-        encode_chunk<PACK>(raw, S[size_t(n) * G + g], qbias[size_t(n) * G + g], tab, lut, w_int, dst, n, kb);
-    }
-    __threadfence();   // operands visible device-wide before the block counts as finished (products fetch them early)
+    const double s = double(__half2float(s_h));
+    return __half_as_ushort(__double2half(j < q ? s * tab.plane_weight[j & 3] : s * tab.centre + double(__half2float(b_h))));
 }
 
-// Groups of 128: everything in one pass.  A group is 16 chunks = 16 consecutive lanes, each holding
-// its chunk in registers: range by shuffles, S and qbias by the group's first lane, then the encoding.
-template <bool PACK>
-__global__ void __launch_bounds__(256) rtn_fused128_kernel(const __half *__restrict__ W, QuantTable tab,
-                                                           __half *__restrict__ S, __half *__restrict__ qbias,
-                                                           uint8_t *__restrict__ w_int, const View dst)
+// the integer by its definition
+__device__ __noinline__ uint32_t exact_int(uint32_t w16, __half b_h, __half s_h, double top)
+{
+    const double w = double(__half2float(__ushort_as_half(uint16_t(w16)))), b = double(__half2float(b_h)), s = double(__half2float(s_h));
+    if (!(s > 0.0)) return 0u;                         // a constant group (or a NaN scale)
+    const double r = rint(__ddiv_rn(w - b, s));        // the subtraction is exact in fp64
+    return uint32_t(fmin(fmax(r, 0.0), top));
+}
+
+// Per-group constants of the integer decision.  t = (W - qbias)/S is evaluated as ONE fp32 fused multiply-add onto a
+// constant that carries 2^23 / 2^FR, one half and a margin of e ulps: the result's mantissa then holds t + 1/2 + margin
+// in fixed point with FR fraction bits, its integer part being the rounded quotient, unless the fraction is below
+// 2 e -- then the quotient lies within the error bound of a rounding boundary (exact ties do) and the fp64 definition
+// decides.  Error in units of 2^-FR: 1/2 for the rounding of the result, (|qbias/S| + 257) 2^(FR - 24) for the constant,
+// t 2^(FR - 24) <= 1 for the reciprocal where t is inside the range (beyond it every value clamps to the top).
+template <int FR>
+struct IntDecision {
+    float inv, c;
+    int ceiling;         // bit pattern of "top": everything beyond is the top integer
+    uint32_t doubt;      // fractions below this go to fp64; > 65535: all do
+    __device__ IntDecision(__half s_h, __half b_h, float lo, float hi, double top)
+    {
+        const float sf = __half2float(s_h), bf = __half2float(b_h);
+        constexpr float kOne = float(1 << FR), kBase = 8388608.f / kOne;   // [kBase, 2 kBase): ulp 2^-FR
+        inv = sf > 0.f ? __frcp_rn(sf) : 0.f;   // S = 0: every integer is 0
+        const float far = fabsf(bf) * inv;
+        // (S overflowed, or the range or a weight is not a finite number: leave it to the definition)
+        const bool plain = sf < 65536.f && fabsf(lo) < 65536.f && fabsf(hi) < 65536.f && far < 1048576.f;
+        const int e = plain ? 4 + int(far * (1.f / 256.f)) : 0;
+        doubt = plain ? uint32_t(2 * e) : 0x10000u;
+        c = plain ? fmaf(-bf, inv, kBase + 0.5f + float(e) / kOne) : kBase;
+        if (!plain) inv = 0.f;
+        ceiling = __float_as_int(kBase + float(top) + 0.5f);
+    }
+};
+
+// Integers of the 8 weights of one 16-byte piece, one per byte.
+template <int FR>
+__device__ __forceinline__ uint2 piece_ints(const uint4 raw, const IntDecision<FR> &dec, __half s_h, __half b_h, double top)
+{
+    const uint32_t word[4] = {raw.x, raw.y, raw.z, raw.w};
+    uint32_t bits[8];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&word[j]));
+        bits[2 * j] = uint32_t(min(__float_as_int(fmaf(f.x, dec.inv, dec.c)), dec.ceiling));
+        bits[2 * j + 1] = uint32_t(min(__float_as_int(fmaf(f.y, dec.inv, dec.c)), dec.ceiling));
+    }
+    uint32_t least = 0xffffffffu;   // smallest fraction, two halves
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        uint32_t pair = __byte_perm(bits[2 * j], bits[2 * j + 1], 0x5410u);
+        if (FR == 15) pair &= 0x7fff7fffu;
+        least = __vminu2(least, pair);
+    }
+    if (FR == 15) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) bits[j] <<= 1;   // the integer into byte 2
+    }
+    if (min(least & 0xffffu, least >> 16) < dec.doubt) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const uint32_t frac = FR == 15 ? (bits[j] & 0xffffu) >> 1 : bits[j] & 0xffffu;
+            if (frac < dec.doubt) bits[j] = exact_int(word[j >> 1] >> (16 * (j & 1)), b_h, s_h, top) << 16;
+        }
+    }
+    return make_uint2(__byte_perm(__byte_perm(bits[0], bits[1], 0x0062u), __byte_perm(bits[2], bits[3], 0x0062u), 0x5410u),
+                      __byte_perm(__byte_perm(bits[4], bits[5], 0x0062u), __byte_perm(bits[6], bits[7], 0x0062u), 0x5410u));
+}
+
+// entry t of the table = the code of step-1 integer t with code bit i moved to bit 8 i: the 8 entries of a chunk,
+// shifted by their position and added up, are the chunk's byte of plane i in byte i
+__device__ __forceinline__ uint32_t chunk_planes(const uint2 ints, const uint32_t *lut)
+{
+    uint32_t spread = 0u;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        spread += lut[(ints.x >> (8 * j)) & 0xffu] << j;
+        spread += lut[(ints.y >> (8 * j)) & 0xffu] << (4 + j);
+    }
+    return spread;
+}
+
+// LANES: lanes per group, 4, 2 or 1 for groups of 128, 64 and 32 (one pass; jobs = (row unit, segment), segments
+// fastest); 0 for any other group length L: a block takes the row unit blockIdx.x, ranges first.
+// PACK = false (the search over scale factors wants the integers only): no planes, no fused scales.
+template <int FR, bool PACK, int LANES>
+__global__ void __launch_bounds__(256, 3) rtn_kernel(const __half *__restrict__ W, const __grid_constant__ QuantTable tab, int L,
+                                                  __half *S, __half *qbias, uint8_t *__restrict__ w_int, const View dst)
 {
     __shared__ uint32_t lut[256];
-    load_spread_table(tab, lut);
-    const int kbytes = dst.K / 8;   // a multiple of 16: a half-warp is inside the row or outside
-    const int kb = blockIdx.y * 256 + threadIdx.x;
-    const bool in = kb < kbytes;
-    for (int n = blockIdx.x * kQuantRows; n < min(dst.N, (blockIdx.x + 1) * kQuantRows); ++n) {
-        uint4 raw = make_uint4(0u, 0u, 0u, 0u);
-        if (in) raw = *reinterpret_cast<const uint4 *>(W + size_t(n) * dst.K + size_t(kb) * 8);
-        const __half2 *h2 = reinterpret_cast<const __half2 *>(&raw);
-        float lo, hi;
-        {
-            const float2 f = __half22float2(h2[0]);
-            lo = fminf(f.x, f.y), hi = fmaxf(f.x, f.y);
+    const int lane = threadIdx.x & 31, j = lane >> 2, l = lane & 3, warp = threadIdx.x >> 5;
+    if (PACK) {
+        const uint32_t c = tab.code_of_int[threadIdx.x];
+        lut[threadIdx.x] = (c & 1u) | ((c & 2u) << 7) | ((c & 4u) << 14) | ((c & 8u) << 21);
+    }
+    const int N = dst.N, K = dst.K, G = K / L, q = dst.q;
+    const int segs = (K + kSegment - 1) / kSegment;
+
+    if constexpr (LANES == 0) {   // ranges: a warp per (row, group) of the block's row unit
+        const int u = blockIdx.x, rows = min(kUnitRows, N - u * kUnitRows);
+        for (int un = warp; un < rows * G; un += 8) {
+            const int n = u * kUnitRows + un / G, g = un % G;
+            const __half *w = W + size_t(n) * K + size_t(g) * L;
+            float lo = __half2float(w[0]), hi = lo;
+#pragma unroll 4
+            for (int k = 8 * lane; k < L; k += 256) {   // L is a multiple of 32: whole 16-byte pieces
+                const uint4 raw = *reinterpret_cast<const uint4 *>(w + k);
+                const __half2 *h = reinterpret_cast<const __half2 *>(&raw);
 #pragma unroll
-            for (int j = 1; j < 4; ++j) {
-                const float2 e = __half22float2(h2[j]);
-                lo = fminf(lo, fminf(e.x, e.y));
-                hi = fmaxf(hi, fmaxf(e.x, e.y));
+                for (int i = 0; i < 4; ++i) {
+                    const float2 f = __half22float2(h[i]);
+                    lo = fminf(lo, fminf(f.x, f.y));
+                    hi = fmaxf(hi, fmaxf(f.x, f.y));
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+                hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+            }
+            __half s_h, b_h;
+            range_to_scale(lo, hi, tab, s_h, b_h);
+            if (lane == 0) {
+                S[size_t(n) * G + g] = s_h;
+                qbias[size_t(n) * G + g] = b_h;
+            }
+            if (PACK && lane <= q) {
+                uint16_t *to = lane < q ? dst.alpha_elem(lane, n, g) : dst.z_elem(n, g);
+                *to = fused_scale(s_h, b_h, tab, q, lane);
             }
         }
+    }
+    __syncthreads();
+
+    const PlaneWriter out(dst);
+    const size_t stride = dst.plane_stride();
+    const int units = LANES ? (N + kUnitRows - 1) / kUnitRows : int(blockIdx.x) + 1;   // the walk ends there
+    SegmentWalk at_job(LANES ? (long long)blockIdx.x * 8 + warp : (long long)blockIdx.x * segs + warp, LANES ? (long long)gridDim.x * 8 : 8, segs);
+    uint4 raw[4];
+    auto fetch = [&](const SegmentWalk &w) {
+        const int n = w.u * kUnitRows + j, k = w.seg * kSegment + 32 * l;
+        const bool in = w.u < units && n < N && k < K;
+        const uint4 *src = reinterpret_cast<const uint4 *>(W + size_t(n) * K + k);
 #pragma unroll
-        for (int o = 8; o > 0; o >>= 1) {
-            lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-            hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        for (int c = 0; c < 4; ++c) raw[c] = in ? src[c] : make_uint4(0u, 0u, 0u, 0u);
+    };
+    fetch(at_job);
+    while (at_job.u < units) {
+        const int u = at_job.u, seg = at_job.seg;
+        const int n = u * kUnitRows + j, k = seg * kSegment + 32 * l;
+        const bool in = n < N && k < K;
+        __half s_h, b_h;
+        float lo, hi;
+        if constexpr (LANES > 0) {
+            // the group's range in fp16 (exact); a NaN weight is ignored, but makes the group go by the definition
+            const __half2 *h = reinterpret_cast<const __half2 *>(raw);
+            __half2 lo2 = h[0], hi2 = h[0];
+#pragma unroll
+            for (int i = 1; i < 16; ++i) lo2 = __hmin2(lo2, h[i]), hi2 = __hmax2_nan(hi2, h[i]);
+            __half lo_h = __hmin(__low2half(lo2), __high2half(lo2)), hi_h = __hmax_nan(__low2half(hi2), __high2half(hi2));
+            for (int o = 1; o < LANES; o *= 2) {
+                const __half2 both = __halves2half2(lo_h, hi_h);
+                const uint32_t got = __shfl_xor_sync(0xffffffffu, *reinterpret_cast<const uint32_t *>(&both), o);
+                const __half2 other = *reinterpret_cast<const __half2 *>(&got);
+                lo_h = __hmin(lo_h, __low2half(other)), hi_h = __hmax_nan(hi_h, __high2half(other));
+            }
+            lo = __half2float(lo_h), hi = __half2float(hi_h);
+            float hi_scale = hi;
+            if (__any_sync(0xffffffffu, hi != hi)) {
+                hi2 = h[0];
+#pragma unroll
+                for (int i = 1; i < 16; ++i) hi2 = __hmax2(hi2, h[i]);
+                hi_h = __hmax(__low2half(hi2), __high2half(hi2));
+                for (int o = 1; o < LANES; o *= 2) {
+                    const uint32_t mine = __half_as_ushort(hi_h);
+                    hi_h = __hmax(hi_h, __ushort_as_half(uint16_t(__shfl_xor_sync(0xffffffffu, mine, o))));
+                }
+                hi_scale = __half2float(hi_h);
+            }
+            range_to_scale(lo, hi_scale, tab, s_h, b_h);
+            const int li = l & (LANES - 1);          // this lane inside its group
+            const int g = seg * (4 / LANES) + l / LANES;
+            if (in && li == 0) {
+                S[size_t(n) * G + g] = s_h;
+                qbias[size_t(n) * G + g] = b_h;
+            }
+            if (PACK && in) {   // the group's lanes share out its q + 1 fused scales
+                constexpr int sub = 4 / LANES;
+                const int per = q + 1;
+                uint16_t *tile_scales = reinterpret_cast<uint16_t *>(dst.packed + dst.tile_base(seg >> 2, u) + size_t(q) * 512) +
+                                        (size_t(8 * (seg & 3) + j) * sub + tile_phase(sub, j, l / LANES)) * per;
+                for (int i = li; i <= q; i += LANES) {
+                    uint16_t *to = out.tiled ? tile_scales + i : (i < q ? dst.alpha + (size_t(i) * N + n) * G + g : dst.z + size_t(n) * G + g);
+                    *to = fused_scale(s_h, b_h, tab, q, i);
+                }
+            }
+        } else {
+            const size_t unit = in ? size_t(n) * G + k / L : 0;
+            s_h = S[unit], b_h = qbias[unit];
+            lo = __half2float(b_h);
+            // (a NaN weight in a group that has other numbers shows up here, not in the range)
+            const __half2 *h = reinterpret_cast<const __half2 *>(raw);
+            __half2 hi2 = h[0];
+#pragma unroll
+            for (int i = 1; i < 16; ++i) hi2 = __hmax2_nan(hi2, h[i]);
+            hi = __half2float(__hmax_nan(__low2half(hi2), __high2half(hi2)));
         }
-        // S and qbias by the group's first lane, handed to the other 15; then lanes 0 .. q of the group
-        // each produce one fused scale (alpha_0 .. alpha_{q-1}, z = S centre + qbias) in the same pass.
-        __half s_h = __float2half_rn(0.f), b_h = s_h;
-        const int sub = threadIdx.x & 15;
-        const int g = kb >> 4, G = dst.K / 128;
-        if (sub == 0 && in) {
-            range_to_scale(lo, hi, tab, s_h, b_h);
-            S[size_t(n) * G + g] = s_h;
-            qbias[size_t(n) * G + g] = b_h;
+        const IntDecision<FR> dec(s_h, b_h, lo, hi, tab.top);
+        uint2 ints[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) ints[c] = piece_ints<FR>(raw[c], dec, s_h, b_h, tab.top);
+        at_job.next();
+        fetch(at_job);   // the next job's weights are on their way while this one's planes are put together
+        if (w_int && in) {
+            uint2 *to = reinterpret_cast<uint2 *>(w_int + size_t(n) * K + k);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) to[c] = ints[c];
         }
-        const unsigned pair = uint32_t(__half_as_ushort(s_h)) | (uint32_t(__half_as_ushort(b_h)) << 16);
-        const unsigned got = __shfl_sync(0xffffffffu, pair, (threadIdx.x & 31) & 16);
-        s_h = __ushort_as_half(uint16_t(got & 0xffffu));
-        b_h = __ushort_as_half(uint16_t(got >> 16));
-        if (PACK && in && sub <= dst.q) {
-            const double mult = sub < dst.q ? tab.plane_weight[sub & 3] : tab.centre;
-            const double add = sub < dst.q ? 0.0 : double(__half2float(b_h));
-            const uint16_t v = __half_as_ushort(__double2half(double(__half2float(s_h)) * mult + add));   // exact, rounded once
-            if (sub < dst.q)
-                *dst.alpha_elem(sub, n, g) = v;
-            else
-                *dst.z_elem(n, g) = v;
+        if (PACK) {
+            uint32_t p[4];   // byte i of p[c]: plane i's byte of chunk c
+#pragma unroll
+            for (int c = 0; c < 4; ++c) p[c] = chunk_planes(ints[c], lut);
+            unsigned char *at = out.at(dst, u, seg);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                if (i < q) {
+                    const uint32_t ab = __byte_perm(p[0], p[1], 0x0040u + 0x11u * i), cd = __byte_perm(p[2], p[3], 0x0040u + 0x11u * i);
+                    const uint32_t w = out.word(__byte_perm(ab, cd, 0x5410u));
+                    if (in) *reinterpret_cast<uint32_t *>(at + i * stride) = w;
+                }
+            }
         }
-        if (in) encode_chunk<PACK>(raw, s_h, b_h, tab, lut, w_int, dst, n, kb);
     }
     __threadfence();   // operands visible device-wide before the block counts as finished (products fetch them early)
 }
 
-// One thread per (row, group): the fused scales, written where the destination layout keeps them.
-__global__ void __launch_bounds__(256) rtn_scales_kernel(const __half *__restrict__ S, const __half *__restrict__ qbias,
-                                                         QuantTable tab, const View dst)
+template <int FR>
+static cudaError_t launch_rtn(const __half *w, const QuantTable &tab, __half *s, __half *b, uint8_t *w_int, const View &dst, cudaStream_t st,
+                              bool pack)
 {
-    const int G = dst.G();
-    const size_t t = size_t(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (t >= size_t(dst.N) * G) return;
-    write_scales(S[t], qbias[t], tab, dst, int(t / G), int(t % G));
-    __threadfence();   // as in the encoding kernels
+    const int L = dst.group == 0 ? dst.K : dst.group;
+    const int lanes = (L == 128 || L == 64 || L == 32) ? L / 32 : 0;
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const long long blocks = lanes ? (segment_jobs(dst.N, dst.K) + 7) / 8 : (dst.N + kUnitRows - 1) / kUnitRows;
+    // one pass: as many blocks as the GPU holds, each walking many jobs (the set-up of a block and its closing fence
+    // cost about as much as a job); two passes: a block per row unit
+    const unsigned grid = unsigned(lanes ? (blocks < sms * 3LL ? blocks : sms * 3LL) : blocks);
+    const auto kernel = lanes == 4   ? (pack ? rtn_kernel<FR, true, 4> : rtn_kernel<FR, false, 4>)
+                        : lanes == 2 ? (pack ? rtn_kernel<FR, true, 2> : rtn_kernel<FR, false, 2>)
+                        : lanes == 1 ? (pack ? rtn_kernel<FR, true, 1> : rtn_kernel<FR, false, 1>)
+                                     : (pack ? rtn_kernel<FR, true, 0> : rtn_kernel<FR, false, 0>);
+    kernel<<<grid, 256, 0, st>>>(w, tab, L, s, b, w_int, dst);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_quantize_rtn(const uint16_t *W, int n_bits, double s_factor, const uint8_t *code_of_int /*[256]*/,
@@ -237,29 +314,10 @@ cudaError_t launch_quantize_rtn(const uint16_t *W, int n_bits, double s_factor, 
     tab.top = double((1u << n_bits) - 1u);
     tab.centre = tab.top / 2.0;
     tab.s_factor = s_factor;
-    const int L = dst.group == 0 ? dst.K : dst.group;
-    const size_t units = size_t(dst.N) * dst.G();
     const __half *w = reinterpret_cast<const __half *>(W);
     __half *s = reinterpret_cast<__half *>(S), *b = reinterpret_cast<__half *>(qbias);
-    const dim3 grid(unsigned((dst.N + kQuantRows - 1) / kQuantRows), unsigned((dst.K / 8 + 255) / 256));   // kQuantRows rows per block
-    if (L == 128) {
-        if (pack)
-            rtn_fused128_kernel<true><<<grid, 256, 0, st>>>(w, tab, s, b, w_int, dst);
-        else
-            rtn_fused128_kernel<false><<<grid, 256, 0, st>>>(w, tab, s, b, w_int, dst);
-        return cudaGetLastError();
-    }
-    rtn_range_kernel<<<unsigned((units + 7) / 8), 256, 0, st>>>(w, dst.N, dst.K, L, tab, s, b);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    if (pack)
-        rtn_encode_kernel<true><<<grid, 256, 0, st>>>(w, s, b, L, tab, w_int, dst);
-    else
-        rtn_encode_kernel<false><<<grid, 256, 0, st>>>(w, s, b, L, tab, w_int, dst);
-    e = cudaGetLastError();
-    if (e != cudaSuccess || !pack) return e;
-    rtn_scales_kernel<<<unsigned((units + 255) / 256), 256, 0, st>>>(s, b, tab, dst);
-    return cudaGetLastError();
+    // 16 fraction bits leave 7 integer bits in the mantissa
+    return n_bits <= 7 ? launch_rtn<16>(w, tab, s, b, w_int, dst, st, pack) : launch_rtn<15>(w, tab, s, b, w_int, dst, st, pack);
 }
 
 }  // namespace bcq

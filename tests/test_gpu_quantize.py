@@ -157,3 +157,51 @@ def test_quantize_rtn_rejects_bad_arguments():
         bq.quantize_rtn(d, t16, 4, [0, 1, 2, 2], sc, sc, None, t8, sc, sc, s_factor=0.0)
     with pytest.raises(bq.BcqError):
         bq.quantize_rtn(d, t16, 4, [0, 1, 2, 2], sc, sc, None, t8, None, None)   # canonical needs alpha and z
+
+
+@pytest.mark.parametrize("N,K,q,group,layout,n_bits,b2p,s_factor", [
+    (17, 160, 2, 32, bq.LAYOUT_CANONICAL, 3, [0, 1, 1], 1.0),             # ragged rows and a short last segment
+    (9, 384, 3, 96, bq.LAYOUT_CANONICAL, 5, [0, 1, 1, 2, 2], 0.52),       # groups that straddle segments; many clamped
+    (8, 4128, 1, 0, bq.LAYOUT_CANONICAL, 7, [0] * 7, 1.0),
+    (5, 256, 4, 256, bq.LAYOUT_CANONICAL, 8, [0, 0, 1, 1, 2, 2, 3, 3], 0.7),   # 15 fraction bits
+    (16, 512, 3, 64, bq.LAYOUT_TILED, 8, [0, 0, 0, 1, 1, 1, 2, 2], 1.0),
+    (24, 1024, 4, 32, bq.LAYOUT_TILED, 6, [0, 1, 1, 2, 2, 3], 0.6),
+    (16, 512, 2, 0, bq.LAYOUT_TILED, 4, [0, 0, 1, 1], 1.0),
+    (8, 512, 3, 128, bq.LAYOUT_TILED, 7, [0, 0, 1, 1, 1, 2, 2], 1.0),
+])
+@pytest.mark.parametrize("kind", ["normal", "grid", "offset", "tiny"])
+def test_quantize_rtn_where_the_estimate_does_not_decide(N, K, q, group, layout, n_bits, b2p, s_factor, kind):
+    """Weights on and next to rounding boundaries (a grid of half steps), ranges far away from zero (the offset is
+    thousands of steps), subnormal scales: the integers stay those of the fp64 definition."""
+    rng = np.random.default_rng(N * K + n_bits)
+    if kind == "normal":
+        W = weights(f"q2/{N}x{K}", N, K)
+    elif kind == "grid":
+        W = (rng.integers(0, 2 ** (n_bits + 1) - 1, (N, K)) * 0.5 - 3).astype(np.float16)
+    elif kind == "offset":
+        W = (100.0 + rng.integers(0, 5, (N, K)) * 0.0625).astype(np.float16)
+    else:
+        W = (rng.integers(0, 300, (N, K)) * 2.0 ** -24 + rng.integers(0, 2, (N, 1))).astype(np.float16)
+    S, qb, wi, packed, a, z = run(W, q, group, layout, n_bits, b2p, s_factor)
+    e_wi, e_S, e_qb, e_packed, e_a, e_z, _ = expected(W, q, group, layout, n_bits, b2p, s_factor)
+    assert same(S, e_S) and same(qb, e_qb) and same(wi, e_wi) and same(packed, e_packed)
+    if a is not None:
+        assert same(a, e_a) and same(z, e_z)
+
+
+@pytest.mark.parametrize("group", [32, 128, 0])
+def test_quantize_rtn_weights_that_are_not_numbers(group):
+    """A NaN among finite weights is ignored by the range and becomes integer 0; the others are not disturbed."""
+    N, K = 8, 512
+    W = weights("q/nan", N, K)
+    clean = W.copy()
+    W[3, 77] = np.float16(np.nan)
+    lo = np.nanargmin(W[3, 64:96])
+    clean[3, 77] = W[3, 64 + lo]                      # a value that changes no minimum or maximum
+    S, qb, wi, packed, a, z = run(W, 3, group, bq.LAYOUT_TILED, 4, [0, 1, 2, 2])
+    e_wi, e_S, e_qb, *_ = expected(clean, 3, group, bq.LAYOUT_TILED, 4, [0, 1, 2, 2])
+    assert same(S, e_S) and same(qb, e_qb)
+    wi, e_wi = wi.reshape(N, K), e_wi.reshape(N, K).copy()
+    assert wi[3, 77] == 0
+    e_wi[3, 77] = 0
+    assert np.array_equal(wi, e_wi)
