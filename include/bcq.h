@@ -143,9 +143,9 @@ int bcq_check_desc(const bcq_desc *desc);
 int bcq_plan_default(const bcq_desc *desc, int B, int sm_count, bcq_plan *plan_out);
 
 /* Bytes of workspace the plan needs (0 when k_splits == 1 and the generic kernel).  The
- * workspace holds the split-K partial sums and arrival counts (kernel 1: one 64-bit word per
- * row and column, in which the K splits' sums meet as fixed-point numbers in units of 2^-26;
- * a split's partial sum beyond +-131071 saturates).  It must be zero-filled once
+ * workspace holds the split-K partial sums and arrival counts (one 64-bit word per row and
+ * column, in which the K splits' sums meet as fixed-point numbers in units of 2^-26; a split's
+ * partial sum beyond +-131071, kernel 2 with few splits: beyond more, saturates).  It must be zero-filled once
  * (bcq_workspace_init) before its first use; every call leaves it zero where it has to be, so
  * it can be reused by later calls ON THE SAME STREAM.  Two products in flight at once
  * need two workspaces.  After a call that bcq_poll_status reported as timed out the counters
@@ -268,13 +268,12 @@ int bcq_multi_row_blocks(const bcq_desc *desc, const bcq_plan *plan, const int32
 /*
  * Y[b] = W X[b] for b < B, 1 <= B <= 16; X [B][K], Y [B][N] row-major fp16.  Every column is
  * an independent product (the paper defines batch 1 only; Eq. bcw + Eq. fuse_step3 per column).
- * B == 1 is bcq_gemv.  Tiled layout: by default B >= 4 takes ONE pass over the packed weights
- * for all columns (plan kernel 2, the tensor-core kernel: a weight bit becomes the fp16 value
- * +-alpha of its row and group, the products with x are exact, all sums fp32; the offset term
- * uses the fp32 group sums of x, kept to 22 bits) and B == 2, 3 run the lookup-table kernel on
- * column pairs (plan kernel 1 with tables that hold two columns' sums side by side: one pass
- * over the weights and one 4-byte lookup per weight byte for both columns of a pair; every
- * column is bit-identical to bcq_gemv on it), which is faster there (bcq_plan_default tells
+ * B == 1 is bcq_gemv.  Tiled layout: by default B >= 5 (one scale per row: B >= 2) takes ONE
+ * pass over the packed weights for all columns (plan kernel 2, the tensor-core kernel: the weight
+ * bits select +x or -x, sums of 128 weights in fp32 are scaled by alpha in fp32) and B == 2 .. 4
+ * run the lookup-table kernel on column pairs (plan kernel 1 with tables that hold two columns'
+ * sums side by side: one pass over the weights and one 4-byte lookup per weight byte for both
+ * columns of a pair; every column is bit-identical to bcq_gemv on it; bcq_plan_default tells
  * which).  The workspace depends on B: bcq_workspace_bytes(desc, B, plan).
  * Canonical layout: one pass of the generic kernel for all columns.
  * bcq_gemm_smallbatch_plan takes the decomposition from the caller; a plan with kernel 1 runs

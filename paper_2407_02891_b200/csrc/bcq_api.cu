@@ -56,10 +56,12 @@ int device_sm_count(int *out)
     return BCQ_OK;
 }
 
-// From this many columns on the default plan is the tensor-core kernel.  With the scales in the tiles the
-// lookup-table kernel takes two columns per pass, and two such passes (4 columns) are still faster than one
-// pass of the tensor-core kernel (measured on Llama-2-70B-shaped layers: 1.73 against 2.03 ms per 8 layers).
-constexpr int kSmallBatchMin = 4;
+// From this many columns on the default plan is the tensor-core kernel.  With the scales in the tiles the lookup-table
+// kernel takes two columns per pass, and up to two such passes are the default: every column is then bit-identical to
+// bcq_gemv on it (8192 x 8192, q = 3: 10.9 us at two columns against 18.6; 19.6 and 21.2 at three and four against 18.7).
+// With one scale per row it takes a pass per column (8192 x 8192, two columns: q = 3 21.2 us against 19, q = 2 16.2
+// against 15.8; 4096 x 4096, q = 4: 14.5 against 7.7).
+constexpr int kSmallBatchMin = 2;
 constexpr int kSmallBatchMinPairs = 5;
 // column pairs and the tensor-core kernel exist for groups of 128 (and, the latter, one scale per row); groups of
 // 64 and 32 run the lookup-table kernel column by column
@@ -146,23 +148,23 @@ int plan_lut(const bcq_desc *d, int B, int sm, bcq_plan *out)
     return best < 0 ? BCQ_ERR_UNSUPPORTED_SHAPE : BCQ_OK;
 }
 
-// The same kind of model for the small-batch kernel, fitted to sweeps at 8 and 16 columns over the
-// OPT-30B and Llama-2-70B layer shapes (pick within 0.5 % of the fastest measured plan on average, 3.5 %
-// at worst): a round is one pair of row units per consumer warp; the combine grows with splits x rows x
-// columns.
-long long mma_cost(int U, int W, int rb, int ks, int sm, int B)
+// The same kind of model for the small-batch kernel, fitted to sweeps of decompositions at 4, 8 and 16 columns over 15
+// shapes (2, 3 and 4 planes): its pick is within 1 % of the fastest measured plan on average, 9 % at worst.  A block's
+// (pair of row units, window) jobs run on 16 warps; a round of them costs between its share of the tensor pipe and a
+// whole job; x is staged before the first job, outputs of a split leave by one atomic each, and pairs that warps share
+// are put together at the end.
+double mma_cost(int U, int W, int rb, int ks, int sm, int B, int q, int at_once)
 {
-    const long long per_window = 300, round = 1500, per_pair = 200, per_split = 100, combine = 24;
+    const double job = (B > 8 ? 4570.0 : 2620.0) * q / 3.0 + 540.0, round_weight = 0.33;
+    const double fixed = 2900.0, stage = 27.0, split = 390.0, per_output = 10.0, shared = 560.0, phase = 1450.0;
     const long long waves = (static_cast<long long>(rb) * ks + sm - 1) / sm;
-    const long long wc = (W + ks - 1) / ks;
-    const long long units = (U + rb - 1) / rb;
-    const long long pairs = (units + 1) / 2;
-    long long rounds = (pairs + kMmaWarps - 1) / kMmaWarps;
-    if (rounds < 1) rounds = 1;
-    long long work = rounds * round + pairs * per_pair;
-    if (B > 8) work += work / 2;   // a second MMA per expanded operand
-    long long t = wc * (per_window + work);
-    if (ks > 1) t += per_split * ks + combine * ks * units * B / 8;
+    const int wc = (W + ks - 1) / ks, pairs = ((U + rb - 1) / rb + 1) / 2, jobs = pairs * wc;
+    const bool whole = wc <= at_once;
+    const int rounds = whole ? (jobs + kMmaWarps - 1) / kMmaWarps : (pairs + kMmaWarps - 1) / kMmaWarps * wc;
+    double t = fixed + (round_weight * rounds + (1.0 - round_weight) * jobs / kMmaWarps) * job + stage * wc * B;
+    if (ks > 1) t += split + per_output * pairs * B;
+    if (whole && wc > 1 && (jobs % kMmaWarps != 0 || jobs / kMmaWarps % wc != 0)) t += shared;
+    if (!whole) t += phase * ((wc + at_once - 1) / at_once);
     return waves * t;
 }
 
@@ -170,14 +172,15 @@ int plan_mma(const bcq_desc *d, int sm, int B, bcq_plan *out)
 {
     const int U = d->N / kUnitRows, W = d->K / kWindow;
     const int rb_min = (U + kMmaMaxUnitsPerBlock - 1) / kMmaMaxUnitsPerBlock;
-    long long best = -1;
+    const int at_once = mma_windows_at_once(d->q, d->group != 0, B);
+    double best = -1.0;
     for (int ks = (W + kMaxWindowsPerBlock - 1) / kMaxWindowsPerBlock; ks <= W && ks <= 64; ++ks) {
         for (int k = 0; k <= 16; ++k) {
             for (int j = 0; j <= (k == 1 ? 8 : 0); ++j) {
                 const int rb = k == 0 ? rb_min : (k * sm) / ks - j;
                 if (rb < rb_min || rb < 1 || rb > U || rb > kMaxRowBlocks) continue;
                 if (j > 0 && 10LL * rb * ks < 7LL * sm) continue;
-                const long long c = mma_cost(U, W, rb, ks, sm, B);
+                const double c = mma_cost(U, W, rb, ks, sm, B, d->q, at_once);
                 if (best < 0 || c < best) {
                     best = c;
                     out->kernel = 2;
@@ -245,8 +248,10 @@ size_t plan_workspace(const bcq_desc *d, const bcq_plan *p, int B)
 {
     if (p->k_splits <= 1) return 0;
     // kernel 1 runs one column per launch, or two when the scales live in the tiles
-    if (p->kernel == 1) return lut_workspace_bytes(d->N, (B >= 2 && pairs_ok(d)) ? 2 : 1);
-    if (p->kernel == 2) return kCounterBytes + size_t(p->k_splits) * B * d->N * sizeof(float);
+    if (p->kernel == 1) return split_workspace_bytes(d->N, (B >= 2 && pairs_ok(d)) ? 2 : 1);
+    // kernel 2: one 64-bit word per row and column; the size stays what callers have been told to provide, which is
+    // never less (k_splits >= 2)
+    if (p->kernel == 2) return size_t(16384) + size_t(p->k_splits) * B * d->N * sizeof(float);
     return 0;
 }
 

@@ -16,15 +16,13 @@ constexpr int kGroupsPerWindow = 4; // 128-weight groups in a window
 constexpr int kLutConsumersMax = 23; // consumer warps per block of the lookup-table kernel (some instantiations have fewer)
 constexpr int kLutUnitsPerWarp = 8;  // row units a consumer warp keeps accumulators for
 constexpr int kMaxWindowsPerBlock = 32; // windows one block may walk (bounds the planner's search)
-constexpr int kMmaWarps = 22;        // consumer warps per block of the small-batch kernel
-constexpr int kMmaPairsPerWarp = 4;  // pairs of row units a warp keeps accumulators for
-constexpr int kMmaMaxUnitsPerBlock = 2 * kMmaWarps * kMmaPairsPerWarp;
-constexpr int kMaxRowBlocks = 4096; // small-batch kernel: arrival counters at the head of its workspace
-constexpr size_t kCounterBytes = size_t(kMaxRowBlocks) * sizeof(int);   // small-batch kernel: one counter per row block
+constexpr int kMmaWarps = 16;        // warps per block of the small-batch kernel
+constexpr int kMmaMaxUnitsPerBlock = 176; // row units per block of it (the sums its pairs may have to keep in shared memory)
+constexpr int kMaxRowBlocks = 4096; // row blocks a plan may have
 
-// The lookup-table kernel's split-K workspace: one 64-bit word per row and column (sum and arrival count in
-// one word, see bcq_lut_kernel.cuh); all zero between launches.
-inline size_t lut_workspace_bytes(int N, int cols) { return size_t(cols) * size_t(N) * sizeof(unsigned long long); }
+// The split-K workspace of the lookup-table and the small-batch kernel: one 64-bit word per row and column (sum and
+// arrival count in one word, see bcq_lut_kernel.cuh); all zero between launches.
+inline size_t split_workspace_bytes(int N, int cols) { return size_t(cols) * size_t(N) * sizeof(unsigned long long); }
 // consumer warps and tiles per copy of the instantiation for (q, scales per group?, columns per launch)
 // (sub: scaling units per 128 weights -- 0 = one scale per row, 1, 2 or 4 = groups of 128, 64 or 32)
 int lut_consumer_warps(int q, int sub, int cols);
@@ -162,6 +160,8 @@ cudaError_t launch_lut_multi(const bcq_desc &d, const bcq_plan &plan, const LutO
 cudaError_t launch_dequant_gemv(const bcq_desc &d, const void *packed, const uint16_t *alpha, const uint16_t *z,
                                 const uint16_t *x, uint16_t *y, cudaStream_t st);
 
+// windows of K whose x the small-batch kernel stages at once; blocks with more run in phases
+int mma_windows_at_once(int q, bool grouped, int B);
 cudaError_t launch_mma_gemm(const bcq_desc &d, const bcq_plan &plan, const void *packed, const uint16_t *alpha,
                             const uint16_t *z, const uint16_t *X, uint16_t *Y, int B, void *workspace, cudaStream_t st);
 

@@ -3,48 +3,39 @@
 //
 //   Y[b] = sum_g ( sum_i alpha_i (B_i X[b])_g + z (sum X[b])_g )          (Eq. bcw + Eq. fuse_step3)
 //
-// With several columns the product is a (thin) dense contraction, so the sums go through the
-// tensor cores: mma.sync m16n8k16, fp16 operands, fp32 accumulators, operands in registers.  A
-// weight bit is expanded in registers to the fp16 value +-alpha_i of its (row, group) -- +alpha and
-// -alpha differ in the sign bit only, so a shift, an AND and an XOR turn two bits of a plane word
-// into one operand register -- and x is the other operand, so the products alpha * x are exact and
-// all additions are fp32.  The offset term is one more MMA per tile pair: z times the per-group sums
-// of x, which the loader warps compute in fp32 and pass on as an fp16 (high, low) pair.
-// (The shared-memory-operand tensor path, tcgen05, would need the expanded weights -- 16 times the
-// packed bytes -- written to shared or tensor memory first; with at most 16 columns that costs more
-// than the MMAs themselves, so the register-operand form is used.)
+// With several columns the product is a (thin) dense contraction, so the sums go through the tensor cores: mma.sp
+// m16n8k32, fp16 operands, fp32 accumulators, operands in registers, the weight bits as sparsity metadata (see
+// bcq_mma_core.cuh).  One MMA = 16 weight rows -- two row units, i.e. two tiles of the same window -- x 16 weights x 8
+// columns of X (9 .. 16 columns: a second MMA with the same metadata).  The 128 weights of a scaling unit
+// are 8 MMAs per plane; their sum is scaled in fp32 by the row's alpha.
+// (The shared-memory-operand tensor path, tcgen05, would need the expanded weights -- 16 times the packed bytes --
+// written to shared or tensor memory first; with at most 16 columns that costs more than the MMAs themselves.)
 //
-// Operand roles: A (16 x 16) = 16 weight rows (two row units, i.e. two tiles of the same window)
-// x 16 weights; B (16 x 8) = the same 16 weights of 8 columns of X; C (16 x 8) fp32.  Lane
-// (m = lane / 4, t = lane % 4) holds A elements of rows m and m + 8 only, which is exactly the
-// tile's own distribution: it reads the 16 bytes per plane of tile lane 8 t + m (row m, group t).
-// Because the scale is folded into the operand, the 16 weights of one MMA may come from four
-// different groups (one per t).  The tile stores a row's chunks rotated by two per row (for the
-// batch-1 kernel's bank mapping); the lane undoes that while loading -- word rotation through the
-// load address, the odd half-word through one byte-permute -- so that all rows of an MMA see the
-// same weights k.  X is staged per 512-wide window by two loader warps, already in operand order
-// (one 8-byte shared-memory load per MMA and lane), double buffered.
+// A block owns a range of row units (in pairs) and a range of windows of K.  Its (pair, window) jobs, pair after pair,
+// are dealt to 16 warps in contiguous runs of equal length, so that no warp idles whatever the number of pairs; a pair
+// that two or more warps share is put together through shared memory in a fixed order.  All of the block's x is staged
+// before the first job.  (A decomposition whose x does not fit runs in phases of as many windows as do, whole pairs per
+// warp, sums kept in shared memory between phases.)  Every warp keeps its own ring of slots (one slot = one tile pair =
+// one contiguous piece of memory) filled with bulk async copies.
 //
-// The block structure is that of the batch-1 kernel: one block per SM owns a range of row units and
-// a range of windows; every consumer warp owns a few ring slots (one slot = one tile pair = one
-// contiguous piece of global memory) that it refills itself with bulk async copies; deterministic
-// split-K through fp32 partials and an arrival counter; all waits bounded.
-#include "bcq_async.cuh"
-#include "bcq_internal.cuh"
+// Split K: as in the batch-1 kernel, every output owns one 64-bit word of the workspace, to which a split adds its
+// fixed-point sum and an arrival; whoever completes a word stores y and clears the word.  The result does not depend on
+// the order of arrival.  All waits are bounded.
+//
+// Bound: dispatch of the tensor instruction (9 cycles) and of the half-rate instructions around it (2.5 per MMA: metadata,
+// signs of x, half-words of planes): 16 cycles per MMA and SM sub-partition at up to 8 columns, 13 at 16; then the fixed
+// 4 - 5 us of a launch (x, split-K atomics).  28672 x 8192, q = 3, groups of 128: 71 - 79 us at 8 columns and 103 - 113 at
+// 16 with bits expanded to +-alpha by two instructions per register and whole pairs per warp; 47 and 80 us so.
+#include "bcq_mma_core.cuh"
 
 namespace bcq {
 
-constexpr int kMmaLoaderWarps = 2;
-constexpr int kMmaThreads = (kMmaLoaderWarps + kMmaWarps) * 32;   // 768
-constexpr int kMmaConsumerThreads = kMmaWarps * 32;
+constexpr int kMmaThreads = kMmaWarps * 32;
 constexpr int kMmaSmemBytes = 232448;    // 227 KB: the per-block opt-in maximum
-constexpr int kMmaFixedBytes = 2048;     // barriers and flags
+constexpr int kMmaFixedBytes = 1024;     // barriers and flags
 constexpr int kMmaMaxSlotsPerWarp = 4;
-constexpr int kMmaMaxSlots = kMmaWarps * kMmaMaxSlotsPerWarp;
-constexpr int kXGroupBytes = 264;        // 256 B of operand-ordered x of one (column, group) + 8 B: no bank conflicts
-constexpr int kXRowBytes = 4 * kXGroupBytes;
 
-static_assert(8 * kMmaMaxSlots + 64 <= kMmaFixedBytes, "barrier area");
+static_assert(8 * kMmaWarps * kMmaMaxSlotsPerWarp + 8 <= kMmaFixedBytes, "barrier area");
 
 __device__ int g_mma_status = 0;  // 0, or the code of the wait that ran out (sticky until taken)
 
@@ -54,281 +45,326 @@ struct MmaParams {
     const uint16_t *z;       // per-row scales only: [u][r]
     const __half *X;         // [B][K]
     __half *Y;               // [B][N]
-    float *partial;          // [k_splits][B][N] when k_splits > 1
-    int *counters;           // [row_blocks]
-    int N, K, U, W, B;
-    int row_blocks, k_splits;
+    unsigned long long *accum;   // [B][N] split-K words, all zero between launches; k_splits > 1 only
+    int N, K, B;
+    int u_base, u_rem, w_base, w_rem;   // even partitions: part r starts at r * base + min(r, rem), base + (r < rem) items
+    int split;               // k_splits > 1
+    int phase_windows;       // windows whose x is staged at a time
+    int depth;               // ring slots per warp
+    int x_at, sum_at, ring_at;   // shared memory: constants and x; sums between phases; rings
+    uint32_t ones;           // (1, 1) in fp16: a value known to the compiler would be put into registers again at every use
+    SplitFormat fmt;
 };
 
-enum { kMmaWaitFull = 11, kMmaWaitXReady = 12, kMmaWaitXFree = 13, kMmaWaitDrain = 14 };
-
-__device__ __forceinline__ void mma_16816(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
-                                          uint32_t b1)
-{
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-        : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
-}
+enum { kMmaWaitFull = 11, kMmaWaitDrain = 14 };
 
 // Q planes; GROUPED: scales per (row, group of 128) inside the tiles, else per row in arrays;
 // WIDE: 9..16 columns (two MMAs per step), else at most 8.
 template <int Q, bool GROUPED, bool WIDE>
-__global__ void __launch_bounds__(kMmaThreads, 1) mma_gemm_kernel(const MmaParams p)
+__global__ void __launch_bounds__(kMmaThreads, 1) mma_gemm_kernel(const __grid_constant__ MmaParams p)
 {
     extern __shared__ __align__(128) unsigned char smem[];
     constexpr int T = Q * 512 + (GROUPED ? Q * 64 + 64 : 0);   // bytes of one tile
     constexpr int kSlotBytes = 2 * T;
-    constexpr int BR = WIDE ? 16 : 8;                          // staged columns (zero-filled beyond B)
-    constexpr int kXBufBytes = BR * kXRowBytes;
-    constexpr int PMAX = kMmaPairsPerWarp;
+    constexpr int BR = WIDE ? 16 : 8;
+    constexpr int NA = WIDE ? 8 : 4;                           // accumulators per lane and pair
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-    const int rbi = blockIdx.x % p.row_blocks, ks = blockIdx.x / p.row_blocks;
-    const int u0 = int((long long)rbi * p.U / p.row_blocks), u1 = int((long long)(rbi + 1) * p.U / p.row_blocks);
-    const int w0 = int((long long)ks * p.W / p.k_splits), w1 = int((long long)(ks + 1) * p.W / p.k_splits);
-    const int V = u1 - u0, P = (V + 1) >> 1;   // row units and unit pairs of this block
-    const int nwin = w1 - w0;
+    const int rbi = blockIdx.x, ks = blockIdx.y, U = p.N / kUnitRows;
+    const int u0 = rbi * p.u_base + min(rbi, p.u_rem), w0 = ks * p.w_base + min(ks, p.w_rem);
+    const int V = p.u_base + (rbi < p.u_rem ? 1 : 0), nwin = p.w_base + (ks < p.w_rem ? 1 : 0);
+    const int u1 = u0 + V, P = (V + 1) >> 1;   // row units and unit pairs of this block
+    const bool whole = nwin <= p.phase_windows;   // all of x at once
+    const int D = p.depth;
 
-    // ---- shared memory: [barriers | x operands (2 buffers) | group sums of x (2 buffers) | ring] ----
-    unsigned char *fixed = smem;
-    unsigned char *xs = smem + kMmaFixedBytes;
-    uint32_t *xsum = reinterpret_cast<uint32_t *>(xs + 2 * kXBufBytes);   // [2][BR][4] fp16 (high, low)
-    unsigned char *ring = xs + 2 * kXBufBytes + 2 * BR * 16;
-    constexpr int kRingBytes = kMmaSmemBytes - kMmaFixedBytes - 2 * kXBufBytes - 2 * BR * 16;
-    constexpr int NS = kRingBytes / kSlotBytes < kMmaMaxSlots ? kRingBytes / kSlotBytes : kMmaMaxSlots;
-    constexpr int D = NS / kMmaWarps;   // ring slots per consumer warp
-    static_assert(D >= 1, "ring too small");
+    // ---- shared memory: [barriers | shared pairs' sums | group sums of x | x operands | sums between phases | rings] ----
+    unsigned char *part = smem + kMmaFixedBytes;                               // [run][lane][NA] fp32
+    float *xconst = reinterpret_cast<float *>(smem + p.x_at);                  // [window][segment][column]: sum of x
+    unsigned char *xs = smem + p.x_at + size_t(min(nwin, p.phase_windows)) * 4 * BR * sizeof(float);   // [window][column]
+    unsigned char *between = smem + p.sum_at;                                  // [pair][lane][NA] fp32
+    unsigned char *ring = smem + p.ring_at + warp * D * kSlotBytes;
+    const uint32_t full0 = smem_u32(smem) + 8 * kMmaMaxSlotsPerWarp * warp;
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + 8 * kMmaWarps * kMmaMaxSlotsPerWarp);
 
-    const uint32_t bars = smem_u32(fixed);
-    const uint32_t bar_full = bars;
-    const uint32_t bar_x_ready = bars + 8 * kMmaMaxSlots, bar_x_free = bar_x_ready + 16;
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(fixed + 8 * kMmaMaxSlots + 32);
-    int *s_last = const_cast<int *>(abort_flag) + 1;
-
-    if (warp == 0) {   // one warp initialises the barriers, a few each
-        for (int s = lane; s < kMmaMaxSlots; s += 32) mbar_init(bar_full + 8 * s, 1);
-        if (lane < 2) {
-            mbar_init(bar_x_ready + 8 * lane, BR / 8);   // lane 0 of every loader warp that stages columns
-            mbar_init(bar_x_free + 8 * lane, P < kMmaWarps ? P : kMmaWarps);   // the consumer warps that have jobs
-        }
-        if (lane == 0) *abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    // ---- jobs of this warp: (pair, window) from (pair0, win0) on -----------------------------------------------
+    // Run r belongs to warp (r mod 4) * 4 + r / 4: the runs that get one job more than the others (or the only jobs, where
+    // there are fewer than warps) come at regular distances and would otherwise share a sub-partition's tensor pipe.
+    const int run = (warp & 3) * (kMmaWarps / 4) + (warp >> 2);
+    int total, pair0, win0 = 0;
+    if (whole) {
+        const int jobs = P * nwin, j0 = run * jobs / kMmaWarps;
+        total = (run + 1) * jobs / kMmaWarps - j0, pair0 = j0 / nwin, win0 = j0 - pair0 * nwin;
+    } else {
+        total = warp < P ? (P - warp + kMmaWarps - 1) / kMmaWarps * nwin : 0;
+        pair0 = warp;
     }
-    __syncthreads();
-    // Programmatic dependent launch, as in the batch-1 kernel: weights are constants and may be
-    // fetched before the previous kernel in the stream has finished; X, partials, counters, Y may not.
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-
-    // ---- consumer warps: their jobs (window-major, then their pairs), D of them in flight ---------
-    const int cw = warp - kMmaLoaderWarps;
-    const int mine = (cw >= 0 && P > cw) ? (P - cw + kMmaWarps - 1) / kMmaWarps : 0;   // pairs of this warp per window
-    const int total_jobs = mine * nwin;
-    int issued = 0, consumed = 0, iw = 0, it = 0;
-    auto issue_next = [&](int slot_d) {   // lane 0 of a consumer warp only
-        if (issued < total_jobs) {
-            const int ua = u0 + 2 * (cw + kMmaWarps * it);
-            const size_t tile = size_t(w0 + iw) * p.U + ua;
-            const uint32_t bytes = (ua + 1 < u1) ? kSlotBytes : T;   // the last pair of an odd block is one tile
-            const int s = cw + kMmaWarps * slot_d;
-            const uint32_t full = bar_full + 8 * s;
-            mbar_expect_tx(full, bytes);
-            bulk_g2s(smem_u32(ring + s * kSlotBytes), p.tiles + tile * T, bytes, full);
-            ++issued;
-            if (++it == mine) {
-                it = 0;
-                ++iw;
+    struct Cursor {
+        int pair, win, lo, hi;   // lo .. hi - 1: the windows of the current phase
+    };
+    Cursor next = {pair0, win0, 0, whole ? nwin : p.phase_windows};
+    auto advance = [&](Cursor &c) {
+        if (++c.win == c.hi) {
+            c.win = c.lo;
+            c.pair += whole ? 1 : kMmaWarps;
+            if (!whole && c.pair >= P) {
+                c.pair = warp, c.lo = c.hi, c.hi = min(c.hi + p.phase_windows, nwin);
+                c.win = c.lo;
             }
         }
     };
-    if (cw >= 0 && lane == 0)
-        for (int d0 = 0; d0 < D; ++d0) issue_next(d0);
-
+    int issued = 0, consumed = 0;
+    auto issue_next = [&](int slot) {   // lane 0 only
+        if (issued < total) {
+            const int ua = u0 + 2 * next.pair;
+            const size_t tile = size_t(w0 + next.win) * U + ua;
+            const uint32_t bytes = (ua + 1 < u1) ? kSlotBytes : T;   // the last pair of an odd block is one tile
+            mbar_expect_tx(full0 + 8 * slot, bytes);
+            bulk_g2s(smem_u32(ring + slot * kSlotBytes), p.tiles + tile * T, bytes, full0 + 8 * slot);
+            ++issued;
+            advance(next);
+        }
+    };
+    if (lane == 0) {
+        for (int s = 0; s < D; ++s) mbar_init(full0 + 8 * s, 1);
+        if (tid == 0) *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        // weights are constants and may be fetched before the previous kernel in the stream has finished
+        for (int s = 0; s < D; ++s) issue_next(s);
+    }
+    // Programmatic dependent launch, as in the batch-1 kernel.  X, the split-K words and Y wait for the predecessor.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
-    if (warp < kMmaLoaderWarps) {
-        // ---- loaders: thread (column b, group t) stages its 128 activations of every window ----------
-        // in the order the consumers' B operands want them, plus their fp32 sum as fp16 (high, low).
-        const int b = tid >> 2, t = tid & 3;
-        if (b >= BR) return;
-        for (int wi = 0; wi < nwin; ++wi) {
-            const int buf = wi & 1, use = wi >> 1;
-            uint32_t x2[64];   // x2[j] = (x[2j], x[2j+1]) of the group
-            if (b < p.B) {
-                const uint4 *src = reinterpret_cast<const uint4 *>(p.X + size_t(b) * p.K + size_t(w0 + wi) * kWindow + 128 * t);
-#pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const uint4 v = __ldg(src + j);
-                    x2[4 * j + 0] = v.x, x2[4 * j + 1] = v.y, x2[4 * j + 2] = v.z, x2[4 * j + 3] = v.w;
-                }
-            } else {
-#pragma unroll
-                for (int j = 0; j < 64; ++j) x2[j] = 0u;
-            }
-            if (use > 0 && !mbar_wait<true>(bar_x_free + 8 * buf, (use - 1) & 1, abort_flag, kMmaWaitXFree, &g_mma_status)) break;
-            float sum = 0.f;
-#pragma unroll
-            for (int j = 0; j < 64; ++j) {
-                const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&x2[j]));
-                sum += f.x;
-                sum += f.y;
-            }
-            const __half hi = __float2half_rn(sum), lo = __float2half_rn(sum - __half2float(hi));
-            xsum[(buf * BR + b) * 4 + t] = uint32_t(__half_as_ushort(hi)) | (uint32_t(__half_as_ushort(lo)) << 16);
-            // Operand order.  Consumer lane (., t) keeps in register position k the plane word of chunks
-            // 4L .. 4L+3 of its group, L = (k + t) mod 4; MMA (k, ii) takes, per plane word, the bit pairs
-            // (2ii, 2ii + 16) and (2ii + 1, 2ii + 17): weights 2(ii mod 4) and + 1 of chunks 4L + ii/4 and
-            // 4L + 2 + ii/4.
-            unsigned char *dst = xs + buf * kXBufBytes + b * kXRowBytes + t * kXGroupBytes;
-            static_for<0, 4>([&](auto LL) {
-                constexpr int L = decltype(LL)::value;
-                const int k = (L - t) & 3;
-                static_for<0, 8>([&](auto II) {
-                    constexpr int ii = decltype(II)::value;
-                    const uint32_t lo2 = x2[4 * (4 * L + (ii >> 2)) + (ii & 3)];
-                    const uint32_t hi2 = x2[4 * (4 * L + 2 + (ii >> 2)) + (ii & 3)];
-                    uint2 out;
-                    out.x = __byte_perm(lo2, hi2, 0x5410);   // even weight of both chunks
-                    out.y = __byte_perm(lo2, hi2, 0x7632);   // odd weight of both chunks
-                    *reinterpret_cast<uint2 *>(dst + (k * 8 + ii) * 8) = out;
-                });
-            });
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar_x_ready + 8 * buf);
-        }
-        return;
-    }
-
-    // =============================================================================================
-    // ---- consumers ---------------------------------------------------------------------------------
-    const int ctid = tid - kMmaLoaderWarps * 32;
     const int m = lane >> 2, t = lane & 3;
-    const int lam = 8 * t + m;                 // the tile lane of (row m, group t)
-    const int rot = (m + 1) >> 1;              // the row's chunks are stored rotated by 2 m bytes
-    const uint32_t sel = (m & 1) ? 0x5432u : 0x3210u;
-    int woff[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) woff[k] = lam * 16 + 4 * ((k + t - rot) & 3);
+    struct Ones {   // every non-zero is 1
+        uint32_t v[4];
+        __device__ const uint32_t (&operator()(int, int) const)[4] { return v; }
+    };
+    const Ones unit = {{p.ones, p.ones, p.ones, p.ones}};
+    // chunk pairs 2 t and 2 t + 1 of row m's segment: the tile stores the segment's 16 chunks rotated by 2 m, so they sit
+    // at half-words (2 t - m) mod 8 and (2 t + 1 - m) mod 8 of the row's 16 bytes
+    const int half_lo = m * 16 + 2 * ((2 * t - m) & 7), half_hi = m * 16 + 2 * ((2 * t + 1 - m) & 7);
+    // columns beyond B read a staged column (their accumulators are not stored)
+    const unsigned char *xa0 = xs + (m < p.B ? m : 0) * kXColBytes + t * 16;
+    const unsigned char *xb0 = xs + (m + 8 < p.B ? m + 8 : 0) * kXColBytes + t * 16;
 
-    float acc[PMAX][4], acc_hi[WIDE ? PMAX : 1][4];
+    float acc[NA];
 #pragma unroll
-    for (int pp = 0; pp < PMAX; ++pp)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) acc[pp][e] = 0.f;
-#pragma unroll
-    for (int pp = 0; pp < (WIDE ? PMAX : 1); ++pp)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) acc_hi[pp][e] = 0.f;
-    bool alive = true;
-    int d = 0, fill = 0;   // this warp's ring position: slot cw + kMmaWarps * d, fill number
+    for (int e = 0; e < NA; ++e) acc[e] = 0.f;
 
-    for (int wi = 0; wi < nwin && alive && mine > 0; ++wi) {   // warps without jobs go straight to the end
-        const int buf = wi & 1;
-        if (!mbar_wait<true>(bar_x_ready + 8 * buf, (wi >> 1) & 1, abort_flag, kMmaWaitXReady, &g_mma_status)) {
-            alive = false;
-            break;
+    // outputs of one finished pair: rows m of both units, columns 2 t, 2 t + 1 (and 8 + those)
+    auto emit = [&](int pair) {
+        const int ua = u0 + 2 * pair;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            if (ua + h >= u1) continue;
+            const int n = (ua + h) * kUnitRows + m;
+            unsigned long long before[NA / 2], mine[NA / 2];
+#pragma unroll
+            for (int c = 0; c < NA / 2; ++c) {
+                const int b = 8 * (c >> 1) + 2 * t + (c & 1);
+                const float v = acc[4 * (c >> 1) + 2 * h + (c & 1)];
+                before[c] = 0, mine[c] = 0;
+                if (b < p.B) {
+                    if (p.split) {
+                        mine[c] = split_encode(v, p.fmt);
+                        before[c] = atomicAdd(p.accum + size_t(b) * p.N + n, mine[c]);
+                    } else {
+                        p.Y[size_t(b) * p.N + n] = __float2half_rn(v);
+                    }
+                }
+            }
+            if (p.split) {
+#pragma unroll
+                for (int c = 0; c < NA / 2; ++c) {
+                    const int b = 8 * (c >> 1) + 2 * t + (c & 1);
+                    if (b < p.B && int(before[c] >> p.fmt.count_shift) == p.fmt.arrivals - 1) {
+                        p.Y[size_t(b) * p.N + n] = split_decode(before[c] + mine[c], p.fmt);
+                        p.accum[size_t(b) * p.N + n] = 0;
+                    }
+                }
+            }
         }
-        const unsigned char *xb = xs + buf * kXBufBytes + m * kXRowBytes + t * kXGroupBytes;   // column m (and m + 8)
-        const uint32_t xs_lo = xsum[(buf * BR + m) * 4 + t];
-        const uint32_t xs_hi = WIDE ? xsum[(buf * BR + m + 8) * 4 + t] : 0u;
+    };
 
-        static_for<0, PMAX>([&](auto PP) {
-            constexpr int pp = decltype(PP)::value;
-            if (alive && cw + kMmaWarps * pp < P) {
-                const int s = cw + kMmaWarps * d;
-                if (!mbar_wait(bar_full + 8 * s, fill & 1, abort_flag, kMmaWaitFull, &g_mma_status)) {
-                    alive = false;
-                } else {
-                    ++consumed;
-                    const unsigned char *slot = ring + s * kSlotBytes;
-                    [[maybe_unused]] const int ua = u0 + 2 * (cw + kMmaWarps * pp);
-                    uint32_t Wd[2][Q][4];   // plane words of (row m, group t) of both tiles, rotation undone
-                    uint32_t nb[2][Q];      // (-alpha_i, -alpha_i) as fp16 pairs
-                    uint32_t zz[2];         // (z, z)
+    bool alive = true;
+    int slot = 0, fill = 0, done = 0;
+    Cursor cur = {pair0, win0, 0, whole ? nwin : p.phase_windows};
+    bool began = win0 == 0;   // this warp has the current pair from its first window on
+    for (int lo = 0; lo < nwin; lo += p.phase_windows) {
+        const int nw = min(p.phase_windows, nwin - lo);
+        // ---- stage x of the windows lo .. lo + nw - 1: four threads per (window, column, segment) ----------------
+        if (lo > 0) __syncthreads();   // nobody reads the previous windows' x any more
+#pragma unroll 2
+        for (int base = warp * 32; base < nw * p.B * 16; base += kMmaThreads) {
+            const int task = min(base + lane, nw * p.B * 16 - 1);   // (the count is a multiple of 16)
+            const int st = task & 3, sg = (task >> 2) & 3, wb = task >> 4, w = wb / p.B, b = wb - w * p.B;
+            const uint4 *src = reinterpret_cast<const uint4 *>(p.X + size_t(b) * p.K + size_t(w0 + lo + w) * kWindow + 128 * sg + 32 * st);
+            const uint4 raw[4] = {__ldg(src), __ldg(src + 1), __ldg(src + 2), __ldg(src + 3)};
+            float s = stage_word(raw, xs + size_t(w * p.B + b) * kXColBytes + sg * kXSegBytes, st);
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+            if (st == 0) xconst[(w * 4 + sg) * BR + b] = s;
+        }
+        __syncthreads();
+
+        while (done < total && cur.lo == lo) {
+            if (alive) alive = __all_sync(0xffffffffu, mbar_wait(full0 + 8 * slot, fill & 1, abort_flag, kMmaWaitFull, &g_mma_status));
+            if (!alive) break;
+            ++consumed;
+            if (done > 0 && cur.win == cur.lo) {   // a new pair (this phase)
+#pragma unroll
+                for (int e = 0; e < NA; ++e) acc[e] = 0.f;
+                began = true;
+            }
+            if (lo > 0 && cur.win == lo) {
+                const float *from = reinterpret_cast<const float *>(between) + (cur.pair * 32 + lane) * NA;
+#pragma unroll
+                for (int e = 0; e < NA; ++e) acc[e] = from[e];
+            }
+            const unsigned char *tile = ring + slot * kSlotBytes;
+            const int wl = cur.win - lo;
+            const unsigned char *xa = xa0 + size_t(wl * p.B) * kXColBytes, *xb = xb0 + size_t(wl * p.B) * kXColBytes;
+            const float *xc = xconst + wl * 4 * BR + 2 * t;
+            // (an odd block's last pair has one tile: what the slot holds behind it is read, but rows m + 8 are not stored)
+            [[maybe_unused]] float row_scale[2][Q + 1];
+            if constexpr (!GROUPED) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int u = min(u0 + 2 * cur.pair + h, u1 - 1);
+#pragma unroll
+                    for (int i = 0; i < Q; ++i)
+                        row_scale[h][i] = __half2float(__ushort_as_half(__ldg(p.alpha + (size_t(u) * Q + i) * kUnitRows + m)));
+                    row_scale[h][Q] = __half2float(__ushort_as_half(__ldg(p.z + size_t(u) * kUnitRows + m)));
+                }
+            }
+            float c[Q][4], ch[WIDE ? Q : 1][4];
+            float2 k0 = make_float2(0.f, 0.f), k1 = k0;   // sums of x of columns 2t, 2t + 1; of 8 + those
+            if constexpr (!GROUPED) {
+#pragma unroll
+                for (int g = 0; g < 4; ++g) {
+                    const float2 a = *reinterpret_cast<const float2 *>(xc + g * BR);
+                    k0.x += a.x, k0.y += a.y;
+                    if constexpr (WIDE) {
+                        const float2 b = *reinterpret_cast<const float2 *>(xc + g * BR + 8);
+                        k1.x += b.x, k1.y += b.y;
+                    }
+                }
+            }
+            // acc += scale times the sums of plane i, or z times the sums of x, for the rows of unit h
+            auto scaled = [&](int h, float a, const float (&lo4)[4], const float (&hi4)[4]) {
+                acc[2 * h] = fmaf(a, lo4[2 * h], acc[2 * h]);
+                acc[2 * h + 1] = fmaf(a, lo4[2 * h + 1], acc[2 * h + 1]);
+                if constexpr (WIDE) {
+                    acc[4 + 2 * h] = fmaf(a, hi4[2 * h], acc[4 + 2 * h]);
+                    acc[5 + 2 * h] = fmaf(a, hi4[2 * h + 1], acc[5 + 2 * h]);
+                }
+            };
+            if constexpr (!GROUPED) {
+#pragma unroll
+                for (int i = 0; i < Q; ++i)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        c[i][e] = 0.f;
+                        if constexpr (WIDE) ch[i][e] = 0.f;
+                    }
+            }
+            // (wide, one copy of the body: four are more than the instruction caches hold for 16 warps at different places,
+            // 84.5 -> 87.8 us at 28672 x 8192; up to 8 columns four copies fit and save 2 %)
+#pragma unroll (WIDE ? 1 : 4)
+            for (int g = 0; g < 4; ++g) {
+                uint32_t bits[Q][2];
+#pragma unroll
+                for (int i = 0; i < Q; ++i)
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
-#pragma unroll
-                        for (int i = 0; i < Q; ++i) {
-                            const unsigned char *base = slot + h * T + i * 512;
-                            uint32_t in[4];
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) in[k] = *reinterpret_cast<const uint32_t *>(base + woff[k]);
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) Wd[h][i][k] = __byte_perm(in[k], in[(k + 1) & 3], sel);
-                        }
-                        uint32_t sc[Q + 1];
-                        if constexpr (GROUPED) {
-                            const uint16_t *sp = reinterpret_cast<const uint16_t *>(slot + h * T + Q * 512) + lam * (Q + 1);
-#pragma unroll
-                            for (int i = 0; i <= Q; ++i) sc[i] = sp[i];
-                        } else {
-                            const int u = ua + h;
-#pragma unroll
-                            for (int i = 0; i < Q; ++i) sc[i] = u < u1 ? __ldg(p.alpha + (size_t(u) * Q + i) * kUnitRows + m) : 0;
-                            sc[Q] = u < u1 ? __ldg(p.z + size_t(u) * kUnitRows + m) : 0;
-                        }
-#pragma unroll
-                        for (int i = 0; i < Q; ++i) nb[h][i] = (sc[i] * 0x10001u) ^ 0x80008000u;
-                        zz[h] = sc[Q] * 0x10001u;
+                        const unsigned char *base = tile + i * 512 + g * 128 + (h ? half_hi : half_lo);
+                        const uint32_t a = *reinterpret_cast<const uint16_t *>(base), b = *reinterpret_cast<const uint16_t *>(base + T);
+                        bits[i][h] = __byte_perm(a, b, 0x5410u);
                     }
-                    // The pair is in registers: order those reads before the next copy into the slot
-                    // (generic-proxy reads, then an async-proxy write), then refill the slot.
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                    __syncwarp();
-                    if (lane == 0) issue_next(d);
-
-                    // Independent accumulation chains (an MMA waits for the previous one into the same
-                    // registers): one per plane; folded into the pair's accumulators at the end.
-                    constexpr int NCH = WIDE ? (Q > 1 ? 2 : 1) : Q;
-                    float c[NCH][4], ch[WIDE ? NCH : 1][4];
+                if constexpr (GROUPED) {
+                    k0 = *reinterpret_cast<const float2 *>(xc + g * BR);
+                    if constexpr (WIDE) k1 = *reinterpret_cast<const float2 *>(xc + g * BR + 8);
+                    segment_sums<Q, WIDE, true>(bits, xa + g * kXSegBytes, xb + g * kXSegBytes, unit, c, ch);
+                    // the unit's scales: alpha_i times the signed sums, z times the sum of x
+                    const float zx[4] = {k0.x, k0.y, k0.x, k0.y}, zxh[4] = {k1.x, k1.y, k1.x, k1.y};
 #pragma unroll
-                    for (int j = 0; j < NCH; ++j)
+                    for (int h = 0; h < 2; ++h) {
+                        const unsigned char *sp = tile + h * T + Q * 512 + (8 * g + m) * (2 * (Q + 1));
+                        __align__(8) __half sc[Q + 1];
+                        if constexpr (Q == 3) {
+                            *reinterpret_cast<uint2 *>(sc) = *reinterpret_cast<const uint2 *>(sp);
+                        } else if constexpr (Q == 1) {
+                            *reinterpret_cast<uint32_t *>(sc) = *reinterpret_cast<const uint32_t *>(sp);
+                        } else {
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) c[j][e] = 0.f;
-#pragma unroll
-                    for (int j = 0; j < (WIDE ? NCH : 1); ++j)
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) ch[j][e] = 0.f;
-
-                    // offset term: rows m, m + 8 times (z, z) at k = 2t, 2t + 1; x sums (high, low) there
-                    mma_16816(acc[pp], zz[0], zz[1], 0u, 0u, xs_lo, 0u);
-                    if constexpr (WIDE) mma_16816(acc_hi[pp], zz[0], zz[1], 0u, 0u, xs_hi, 0u);
-
-                    static_for<0, 4>([&](auto KK) {
-                        constexpr int k = decltype(KK)::value;
-                        static_for<0, 8>([&](auto II) {
-                            constexpr int ii = decltype(II)::value;
-                            constexpr int sh0 = 15 - 2 * ii, sh1 = 14 - 2 * ii;
-                            const uint2 xf = *reinterpret_cast<const uint2 *>(xb + (k * 8 + ii) * 8);
-                            uint2 xg = make_uint2(0u, 0u);
-                            if constexpr (WIDE) xg = *reinterpret_cast<const uint2 *>(xb + 8 * kXRowBytes + (k * 8 + ii) * 8);
-#pragma unroll
-                            for (int i = 0; i < Q; ++i) {
-                                const uint32_t a0 = ((Wd[0][i][k] << sh0) & 0x80008000u) ^ nb[0][i];
-                                const uint32_t a1 = ((Wd[1][i][k] << sh0) & 0x80008000u) ^ nb[1][i];
-                                const uint32_t a2 = ((Wd[0][i][k] << sh1) & 0x80008000u) ^ nb[0][i];
-                                const uint32_t a3 = ((Wd[1][i][k] << sh1) & 0x80008000u) ^ nb[1][i];
-                                mma_16816(c[i % NCH], a0, a1, a2, a3, xf.x, xf.y);
-                                if constexpr (WIDE) mma_16816(ch[i % NCH], a0, a1, a2, a3, xg.x, xg.y);
-                            }
-                        });
-                    });
-#pragma unroll
-                    for (int j = 0; j < NCH; ++j)
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            acc[pp][e] += c[j][e];
-                            if constexpr (WIDE) acc_hi[pp][e] += ch[j][e];
+                            for (int i = 0; i <= Q; ++i) sc[i] = reinterpret_cast<const __half *>(sp)[i];
                         }
-                }
-                if (++d == D) {
-                    d = 0;
-                    ++fill;
+                        scaled(h, __half2float(sc[Q]), zx, zxh);
+#pragma unroll
+                        for (int i = 0; i < Q; ++i) scaled(h, __half2float(sc[i]), c[i], ch[WIDE ? i : 0]);
+                    }
+                } else {
+                    segment_sums<Q, WIDE, false>(bits, xa + g * kXSegBytes, xb + g * kXSegBytes, unit, c, ch);
                 }
             }
-        });
-        __syncwarp();
-        if (lane == 0) mbar_arrive(bar_x_free + 8 * buf);
+            if constexpr (!GROUPED) {
+                const float zx[4] = {k0.x, k0.y, k0.x, k0.y}, zxh[4] = {k1.x, k1.y, k1.x, k1.y};
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    scaled(h, row_scale[h][Q], zx, zxh);
+#pragma unroll
+                    for (int i = 0; i < Q; ++i) scaled(h, row_scale[h][i], c[i], ch[WIDE ? i : 0]);
+                }
+            }
+            // the slot has been read: order those reads before the next copy into it, then refill it
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) issue_next(slot);
+            if (++slot == D) {
+                slot = 0;
+                ++fill;
+            }
+            ++done;
+            if (cur.win == nwin - 1) {
+                if (began) {
+                    emit(cur.pair);
+                } else {   // the end of a pair that an earlier warp began
+                    float *to = reinterpret_cast<float *>(part) + (run * 32 + lane) * NA;
+#pragma unroll
+                    for (int e = 0; e < NA; ++e) to[e] = acc[e];
+                }
+            } else if (!whole && cur.win == lo + nw - 1) {   // more windows of the pair in a later phase
+                float *to = reinterpret_cast<float *>(between) + (cur.pair * 32 + lane) * NA;
+#pragma unroll
+                for (int e = 0; e < NA; ++e) to[e] = acc[e];
+            }
+            advance(cur);
+        }
+    }
+
+    // ---- pairs that several warps share: the warp with the first window adds the others' sums up, in the runs' order ----
+    if (whole) {
+        const bool open = done == total && total > 0 && cur.win != 0;   // this warp's last pair is not finished
+        if (alive && open && !began) {
+            float *to = reinterpret_cast<float *>(part) + (run * 32 + lane) * NA;
+#pragma unroll
+            for (int e = 0; e < NA; ++e) to[e] = acc[e];
+        }
+        __syncthreads();
+        if (alive && open && began) {
+            const int jobs = P * nwin, end = (cur.pair + 1) * nwin;
+            for (int c = run + 1; c < kMmaWarps; ++c) {
+                const int s = c * jobs / kMmaWarps, e1 = (c + 1) * jobs / kMmaWarps;
+                if (s >= end) break;
+                if (s == e1) continue;
+                const float *from = reinterpret_cast<const float *>(part) + (c * 32 + lane) * NA;
+#pragma unroll
+                for (int e = 0; e < NA; ++e) acc[e] += from[e];
+            }
+            if (!*abort_flag) emit(cur.pair);
+        }
     }
 
     // Gave up on a wait: copies this warp started may still be in flight.  See them land (bounded)
@@ -336,73 +372,52 @@ __global__ void __launch_bounds__(kMmaThreads, 1) mma_gemm_kernel(const MmaParam
     if (!alive && lane == 0) {
         for (int j = consumed; j < issued; ++j) {
             bool landed = false;
-            for (int itr = 0; itr < kSpinLimit && !landed; ++itr)
-                landed = mbar_try_wait(bar_full + 8 * (cw + kMmaWarps * (j % D)), uint32_t((j / D) & 1));
+            for (int itr = 0; itr < kSpinLimit && !landed; ++itr) {
+                landed = mbar_test_wait(full0 + 8 * (j % D), uint32_t((j / D) & 1));
+                if (!landed) __nanosleep(32);
+            }
             if (!landed) atomicExch(&g_mma_status, int(kMmaWaitDrain));
-        }
-    }
-
-    // ---- store: lane (m, t) holds rows m of both units for columns 2t, 2t+1 (and 8 + those) -------
-    float *partial = p.k_splits > 1 ? p.partial + size_t(ks) * p.B * p.N : nullptr;
-    auto put = [&](int b, int n, float v) {
-        if (b < p.B) {
-            if (partial)
-                partial[size_t(b) * p.N + n] = v;
-            else
-                p.Y[size_t(b) * p.N + n] = __float2half_rn(v);
-        }
-    };
-#pragma unroll
-    for (int pp = 0; pp < PMAX; ++pp) {
-        if (cw + kMmaWarps * pp < P) {
-            const int ua = u0 + 2 * (cw + kMmaWarps * pp);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                if (ua + h < u1) {
-                    const int n = (ua + h) * kUnitRows + m;
-                    put(2 * t, n, acc[pp][2 * h]);
-                    put(2 * t + 1, n, acc[pp][2 * h + 1]);
-                    if constexpr (WIDE) {
-                        put(8 + 2 * t, n, acc_hi[pp][2 * h]);
-                        put(9 + 2 * t, n, acc_hi[pp][2 * h + 1]);
-                    }
-                }
-            }
-        }
-    }
-
-    // ---- split-K: the last block to arrive for this row block adds the partials in fixed order --
-    if (p.k_splits > 1) {
-        __threadfence();
-        named_barrier(2, kMmaConsumerThreads);
-        if (ctid == 0) {
-            const int old = atomicAdd(p.counters + rbi, 1);
-            *s_last = (old == p.k_splits - 1);
-        }
-        named_barrier(2, kMmaConsumerThreads);
-        if (*s_last) {
-            __threadfence();
-            const int R = V * kUnitRows;
-            for (int idx = ctid; idx < p.B * R; idx += kMmaConsumerThreads) {
-                const int b = idx / R, n = u0 * kUnitRows + idx % R;
-                float v = 0.f;
-                for (int k0 = 0; k0 < p.k_splits; k0 += 8) {
-                    float part[8];
-#pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        part[k] = (k0 + k < p.k_splits) ? __ldcg(p.partial + (size_t(k0 + k) * p.B + b) * p.N + n) : 0.f;
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) v += part[k];
-                }
-                p.Y[size_t(b) * p.N + n] = __float2half_rn(v);
-            }
-            if (ctid == 0) p.counters[rbi] = 0;
         }
     }
 }
 
+// Shared memory of one launch: where things lie, how many windows' x is staged at a time and how deep the rings are.
+struct MmaLayout {
+    int phase_windows, depth, x_at, sum_at, ring_at;
+};
+static MmaLayout mma_layout(int q, bool grouped, int B, int windows, int pairs)
+{
+    const int slot = 2 * (q * 512 + (grouped ? (q + 1) * 64 : 0)), wide = B > 8, acc_bytes = wide ? 32 : 16, br = wide ? 16 : 8;
+    const int x_window = B * kXColBytes + 4 * br * int(sizeof(float));
+    MmaLayout l;
+    l.x_at = kMmaFixedBytes + kMmaWarps * 32 * acc_bytes;
+    const int room = kMmaSmemBytes - l.x_at - 128;   // (the rings start at a multiple of 128)
+    const int fit = (room - 2 * kMmaWarps * slot) / x_window;   // two slots per warp at least
+    int sums = 0;
+    if (windows <= fit) {
+        l.phase_windows = windows;
+    } else {   // phases: the pairs' sums between them, and one slot per warp if two leave no room for x
+        sums = pairs * 32 * acc_bytes;
+        int x_room = room - sums - 2 * kMmaWarps * slot;
+        if (x_room < x_window) x_room = room - sums - kMmaWarps * slot;
+        l.phase_windows = x_room / x_window;
+        if (l.phase_windows > windows - 1) l.phase_windows = windows - 1;   // (phases and pairs shared by warps exclude each other)
+    }
+    l.sum_at = l.x_at + l.phase_windows * x_window;
+    l.ring_at = (l.sum_at + sums + 127) / 128 * 128;
+    l.depth = (kMmaSmemBytes - l.ring_at) / (kMmaWarps * slot);
+    if (l.depth > kMmaMaxSlotsPerWarp) l.depth = kMmaMaxSlotsPerWarp;
+    return l;
+}
+int mma_windows_at_once(int q, bool grouped, int B)
+{
+    int w = 1;
+    while (w < kMaxWindowsPerBlock && mma_layout(q, grouped, B, w + 1, 1).phase_windows == w + 1) ++w;
+    return w;
+}
+
 template <int Q, bool GROUPED, bool WIDE>
-static cudaError_t launch_mma_q(const MmaParams &prm, cudaStream_t st)
+static cudaError_t launch_mma_q(const MmaParams &prm, dim3 grid, cudaStream_t st)
 {
     static bool configured[64] = {};   // the shared-memory opt-in is per function and per device
     int dev = 0;
@@ -414,7 +429,7 @@ static cudaError_t launch_mma_q(const MmaParams &prm, cudaStream_t st)
         if (dev >= 0 && dev < 64) configured[dev] = true;
     }
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(prm.row_blocks * prm.k_splits);
+    cfg.gridDim = grid;
     cfg.blockDim = dim3(kMmaThreads);
     cfg.dynamicSmemBytes = kMmaSmemBytes;
     cfg.stream = st;
@@ -427,37 +442,44 @@ static cudaError_t launch_mma_q(const MmaParams &prm, cudaStream_t st)
 }
 
 template <int Q>
-static cudaError_t launch_mma_sel(const MmaParams &prm, bool grouped, cudaStream_t st)
+static cudaError_t launch_mma_sel(const MmaParams &prm, bool grouped, dim3 grid, cudaStream_t st)
 {
     const bool wide = prm.B > 8;
-    if (grouped) return wide ? launch_mma_q<Q, true, true>(prm, st) : launch_mma_q<Q, true, false>(prm, st);
-    return wide ? launch_mma_q<Q, false, true>(prm, st) : launch_mma_q<Q, false, false>(prm, st);
+    if (grouped) return wide ? launch_mma_q<Q, true, true>(prm, grid, st) : launch_mma_q<Q, true, false>(prm, grid, st);
+    return wide ? launch_mma_q<Q, false, true>(prm, grid, st) : launch_mma_q<Q, false, false>(prm, grid, st);
 }
 
 cudaError_t launch_mma_gemm(const bcq_desc &d, const bcq_plan &plan, const void *packed, const uint16_t *alpha,
                             const uint16_t *z, const uint16_t *X, uint16_t *Y, int B, void *workspace, cudaStream_t st)
 {
-    MmaParams prm;
+    MmaParams prm = {};
     prm.tiles = static_cast<const uint8_t *>(packed);
     prm.alpha = alpha;   // used with per-row scales only
     prm.z = z;
     prm.X = reinterpret_cast<const __half *>(X);
     prm.Y = reinterpret_cast<__half *>(Y);
-    prm.counters = static_cast<int *>(workspace);
-    prm.partial = workspace ? reinterpret_cast<float *>(static_cast<unsigned char *>(workspace) + kCounterBytes) : nullptr;
+    prm.accum = static_cast<unsigned long long *>(workspace);
     prm.N = d.N;
     prm.K = d.K;
-    prm.U = d.N / kUnitRows;
-    prm.W = d.K / kWindow;
     prm.B = B;
-    prm.row_blocks = plan.row_blocks;
-    prm.k_splits = plan.k_splits;
+    const int U = d.N / kUnitRows, W = d.K / kWindow;
+    prm.u_base = U / plan.row_blocks, prm.u_rem = U % plan.row_blocks;
+    prm.w_base = W / plan.k_splits, prm.w_rem = W % plan.k_splits;
+    prm.ones = 0x3C003C00u;
+    prm.split = plan.k_splits > 1;
+    prm.fmt = split_format(plan.k_splits);
     const bool grouped = d.group != 0;
+    const int windows = prm.w_base + (prm.w_rem ? 1 : 0), pairs = (prm.u_base + (prm.u_rem ? 1 : 0) + 1) / 2;
+    const MmaLayout l = mma_layout(d.q, grouped, B, windows, pairs);
+    if (l.phase_windows < 1 || l.depth < 1) return cudaErrorInvalidValue;
+    prm.phase_windows = l.phase_windows, prm.depth = l.depth;
+    prm.x_at = l.x_at, prm.sum_at = l.sum_at, prm.ring_at = l.ring_at;
+    const dim3 grid(plan.row_blocks, plan.k_splits);
     switch (d.q) {
-        case 1: return launch_mma_sel<1>(prm, grouped, st);
-        case 2: return launch_mma_sel<2>(prm, grouped, st);
-        case 3: return launch_mma_sel<3>(prm, grouped, st);
-        case 4: return launch_mma_sel<4>(prm, grouped, st);
+        case 1: return launch_mma_sel<1>(prm, grouped, grid, st);
+        case 2: return launch_mma_sel<2>(prm, grouped, grid, st);
+        case 3: return launch_mma_sel<3>(prm, grouped, grid, st);
+        case 4: return launch_mma_sel<4>(prm, grouped, grid, st);
     }
     return cudaErrorInvalidValue;
 }

@@ -342,6 +342,32 @@ def test_lookup_kernel_on_column_pairs(N, K, q, rb, ks, B):
         assert np.array_equal(y1.cpu().numpy().view(np.uint16), Yh[b].view(np.uint16))
 
 
+@pytest.mark.parametrize("N,K,q,group,rb,ks,B", [
+    (1408, 16384, 4, 128, 1, 1, 16),   # phases: 176 units and 32 windows in one block, one ring slot per warp
+    (1400, 8704, 4, 0, 1, 1, 9),       # phases of unequal length, an odd number of units, scales per row
+    (24, 1536, 2, 0, 1, 1, 16),        # six jobs on sixteen warps: every pair is shared
+    (8, 2560, 3, 128, 1, 1, 3),        # one unit, five windows
+    (272, 3584, 1, 128, 1, 1, 8),      # 17 pairs x 7 windows: runs that end inside a pair
+    (640, 4608, 3, 128, 5, 9, 11),     # nine arrivals per word
+])
+def test_small_batch_kernel_shares_pairs_and_phases(N, K, q, group, rb, ks, B):
+    """Every way the (pair, window) jobs can fall on the warps.  Products are exact, sums fp32: what is left is one rounding
+    to fp16 (2^-11 of the value) and sums of K fp32 terms, far below the other half of the bound."""
+    p, codes, alpha, z, X = make_layer(f"share/{N}x{K}q{q}", N, K, q, group, B)
+    ref = oracle.forward_planes(p, alpha, z, X, group)
+    L = gpu_layer(N, K, q, group, bq.LAYOUT_TILED, codes, alpha, z)
+    plan = bq.Plan(2, rb, ks, 0)
+    ws = bq.new_workspace(L.d, B, plan)
+    Y = torch.full((B, N), float("nan"), dtype=torch.float16, device=DEV)
+    for _ in range(2):
+        bq.gemm_smallbatch_plan(L.d, plan, L.packed, L.alpha, L.z, dev(X), Y, B, ws)
+    torch.cuda.synchronize()
+    bq.poll_status()
+    assert rel_err(Y.cpu().numpy(), ref) <= 2.0 ** -10
+    if ws is not None:
+        assert not ws.any()                # every word is cleared again
+
+
 def test_small_batch_kernel_structured_inputs():
     """Unit activations pick out single weights: exact values, every (row, k) position distinguishable."""
     N, K, q, group, B = 64, 1024, 3, 128, 16
