@@ -110,8 +110,8 @@ typedef struct bcq_desc {
     int32_t layout;
 } bcq_desc;
 
-/* How a product is decomposed over the GPU.  kernel: 0 = generic (one warp per row; any valid
- * shape, either layout), 1 = lookup-table kernel (tiled layout, one or two columns per launch),
+/* How a product is decomposed over the GPU.  kernel: 0 = any valid shape, either layout,
+ * no workspace, 1 = lookup-table kernel (tiled layout, one or two columns per launch),
  * 2 = tensor-core small-batch kernel (tiled layout, 2..16 columns per launch); kernels 1 and 2
  * are launched as row_blocks x k_splits thread blocks; k_splits > 1 needs the workspace.
  * Limits: at most 184 (kernel 1; 160 for q = 4 with two columns per launch) or 176 (kernel 2)
@@ -275,7 +275,7 @@ int bcq_multi_row_blocks(const bcq_desc *desc, const bcq_plan *plan, const int32
  * sums side by side: one pass over the weights and one 4-byte lookup per weight byte for both
  * columns of a pair; every column is bit-identical to bcq_gemv on it; bcq_plan_default tells
  * which).  The workspace depends on B: bcq_workspace_bytes(desc, B, plan).
- * Canonical layout: one pass of the generic kernel for all columns.
+ * Canonical layout: one pass over the planes for all columns (plan kernel 0, no workspace).
  * bcq_gemm_smallbatch_plan takes the decomposition from the caller; a plan with kernel 1 runs
  * the lookup-table kernel on two columns at a time when the scales live in the tiles (group
  * 128: ceil(B/2) passes) and column by column otherwise (one scale per row: B passes).

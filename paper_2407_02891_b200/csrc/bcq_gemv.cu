@@ -1,6 +1,6 @@
 // The BCQ product  y = sum_g ( sum_i alpha_i (B_i x)_g + z (sum x)_g )  (Eq. bcw + Eq. fuse_step3),
-// generic form: one warp per output row, direct sign arithmetic, any valid shape, either layout,
-// batch 1..16.  The slow, always-available path; the batch-1 hot path is in bcq_lut.cu.
+// plan kernel 0: the canonical layout goes to bcq_canon.cu; the tiled layout (explicit plans only) to the generic form
+// below, one warp per output row, direct sign arithmetic, batch 1..16, which the tests hold the other kernels against.
 #include "bcq_internal.cuh"
 
 namespace bcq {
@@ -59,6 +59,7 @@ __global__ void __launch_bounds__(256) generic_kernel(const View v, const __half
 cudaError_t launch_generic(const bcq_desc &d, const void *packed, const uint16_t *alpha, const uint16_t *z,
                            const uint16_t *X, uint16_t *Y, int B, cudaStream_t st)
 {
+    if (d.layout == BCQ_LAYOUT_CANONICAL) return launch_canon(d, packed, alpha, z, X, Y, B, st);
     const int warps = 8;
     dim3 grid((d.N + warps - 1) / warps), block(32 * warps);
     const View v = make_view(d, packed, alpha, z);

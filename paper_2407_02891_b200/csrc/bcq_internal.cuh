@@ -139,6 +139,9 @@ cudaError_t launch_pack(const uint8_t *codes, const uint16_t *alpha_in, const ui
 cudaError_t launch_permute_planes(const View &src, const View &dst, cudaStream_t st);
 cudaError_t launch_permute_scales(const View &src, const View &dst, cudaStream_t st);
 
+// any canonical shape, any scaling unit, 1..16 columns
+cudaError_t launch_canon(const bcq_desc &d, const void *packed, const uint16_t *alpha, const uint16_t *z, const uint16_t *X, uint16_t *Y, int B,
+                         cudaStream_t st);
 cudaError_t launch_generic(const bcq_desc &d, const void *packed, const uint16_t *alpha, const uint16_t *z,
                            const uint16_t *X, uint16_t *Y, int B, cudaStream_t st);
 cudaError_t launch_lut_gemv(const bcq_desc &d, const bcq_plan &plan, const void *packed, const uint16_t *alpha,

@@ -173,6 +173,34 @@ LUT_SHAPES = [(1024, 1024, 3, 128), (8, 512, 3, 128), (296, 2048, 3, 128), (1000
               (64, 1024, 1, 0), (2304, 9216, 2, 0)]
 
 
+@pytest.mark.parametrize("N,K,q,group,B", [
+    (1, 32, 1, 32, 1),          # one row, one word
+    (17, 96, 3, 32, 2),         # a row beyond the first sixteen; a segment of three words
+    (33, 544, 2, 0, 16),        # two windows, the second a single word; K split over a cluster of two
+    (40, 480, 4, 96, 5),        # scaling units of three words that straddle segments
+    (23, 1120, 3, 160, 1),
+    (16, 2048, 3, 64, 9),
+    (300, 11008, 3, 128, 1),    # 22 windows over eight blocks
+    (48, 11008, 2, 256, 16),    # phases: 16 columns' x does not fit at once
+    (5000, 1024, 3, 128, 4),    # more 16-row blocks than two per SM
+    (64, 3072, 1, 3072, 3),     # one scaling unit, given as a group
+])
+def test_canonical_products(N, K, q, group, B):
+    """Every scaling-unit form, row and K remainder, cluster split and phase of the canonical kernel.  The bound: one
+    rounding to fp16 (2^-11 of the value) plus fp32 sums, far below the other half."""
+    p, codes, alpha, z, X = make_layer(f"canon/{N}x{K}q{q}g{group}", N, K, q, group, B)
+    ref = oracle.forward_planes(p, alpha, z, X, group)
+    L = gpu_layer(N, K, q, group, bq.LAYOUT_CANONICAL, codes, alpha, z)
+    Y = torch.full((B, N), float("nan"), dtype=torch.float16, device=DEV)
+    bq.gemm_smallbatch(L.d, L.packed, L.alpha, L.z, dev(X), Y, B, None)
+    torch.cuda.synchronize()
+    assert rel_err(Y.cpu().numpy(), ref) <= 2.0 ** -10
+    Y2 = torch.zeros_like(Y)
+    bq.gemm_smallbatch(L.d, L.packed, L.alpha, L.z, dev(X), Y2, B, None)
+    torch.cuda.synchronize()
+    assert torch.equal(Y.view(torch.int16), Y2.view(torch.int16))
+
+
 @pytest.mark.parametrize("N,K,q,group", LUT_SHAPES)
 def test_gemv_lut_kernel_default_plan(N, K, q, group):
     p, codes, alpha, z, x = make_layer(f"lut/{N}x{K}", N, K, q, group)
