@@ -28,7 +28,8 @@
 namespace bcq {
 
 constexpr int kSearchThreads = 512;      // 16 warps form the operand tiles (latency-bound with fewer)
-constexpr int kSearchBlock = kSearchThreads + 32;   // + the warp that issues the MMAs
+constexpr int kSearchFormers = kSearchThreads / 32;
+constexpr int kSearchBlock = kSearchThreads + 64;   // + the warp that issues the MMAs and the one that starts the copies
 constexpr int kSearchRows = 128;        // rows of W per block = M of the MMA
 constexpr int kSearchKTile = 64;        // weights along K per stage: 128 bytes of fp16, one swizzle row
 constexpr int kSearchMaxCand = 4;       // candidates (accumulators) per block
@@ -86,27 +87,12 @@ __device__ __forceinline__ bool search_wait(uint32_t bar, uint32_t parity, volat
 {
     for (int it = 0; it < kSearchSpin; ++it) {
         if (mbar_test_wait(bar, parity)) return true;
-        __nanosleep(64);
+        if (it >= 8) __nanosleep(64);
         if ((it & 255) == 255 && *abort_flag) return false;
     }
     *abort_flag = 1;
     atomicExch(&g_search_status, code);
     return false;
-}
-
-// all forming threads take the same decision (a wait that gives up must not split them at a barrier)
-__device__ __forceinline__ bool formers_all(bool ok)
-{
-    uint32_t out;
-    asm volatile(
-        "{\n\t.reg .pred p, q;\n\t"
-        "setp.ne.u32 q, %1, 0;\n\t"
-        "barrier.cta.red.and.pred p, 1, %2, q;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(out)
-        : "r"(ok ? 1u : 0u), "n"(kSearchThreads)
-        : "memory");
-    return out != 0;
 }
 
 // one box of a tiled tensor map into shared memory, completion counted in bytes on an mbarrier (x: the
@@ -165,8 +151,8 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
         mbar_init(bar0, 1);
         mbar_init(bar0 + 8, 1);
         mbar_init(bar0 + 16, 1);
-        mbar_init(bar0 + 24, 1);
-        mbar_init(bar0 + 32, 1);
+        mbar_init(bar0 + 24, kSearchFormers);
+        mbar_init(bar0 + 32, kSearchFormers);
         for (int i = 5; i < 9; ++i) mbar_init(bar0 + 8 * i, 1);
         abort_s = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -185,7 +171,7 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
 
     const int ktiles = p.K / kSearchKTile;
     bool alive = true;
-    if (warp == kSearchThreads / 32) {
+    if (warp == kSearchFormers) {
         // ---- the issuing warp: per slice, wait until the stage is full, issue the slice's MMAs, hand the stage back ----
         for (int kt = 0; kt < ktiles && alive; ++kt) {
             const int s = kt & 1;
@@ -210,6 +196,40 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
             }
             __syncwarp();
         }
+    } else if (warp == kSearchFormers + 1) {
+        // ---- the copying warp: W and W_int a slice ahead (their stage is read again when every forming warp has finished the
+        // slice before), X as soon as the tensor cores have let go of the stage ----
+        if (lane == 0) {
+            const int row0 = blockIdx.x * kSearchRows, irow0 = int(blockIdx.z) * p.N + row0;   // W_int of the scale factors: one matrix of gridDim.z * N rows
+            int x_started = -1, w_started = -1;
+            auto start_w = [&](int kt) {
+                const uint32_t to = base + uint32_t(kt & 1) * stage_bytes + a_bytes + x_bytes, bar = bar0 + 56 + 8 * (kt & 1);
+                mbar_expect_tx(bar, kSearchWTile + kSearchITile);
+                tma_box_2d(to, &wmap, kt * kSearchKTile, row0, bar);
+                tma_box_2d(to + kSearchWTile, &imap, kt * kSearchKTile, irow0, bar);
+                w_started = kt;
+            };
+            start_w(0);
+            for (int kt = 0; kt < ktiles && alive; ++kt) {
+                if (kt + 1 < ktiles) {
+                    if (kt > 0 && !search_wait(bar0 + 24 + 8 * ((kt - 1) & 1), uint32_t(((kt - 1) >> 1) & 1), abort_flag, 6)) {
+                        alive = false;
+                        break;
+                    }
+                    start_w(kt + 1);
+                }
+                if (kt >= 2 && !search_wait(bar0 + 8 * (kt & 1), uint32_t(((kt >> 1) - 1) & 1), abort_flag, 7)) {
+                    alive = false;
+                    break;
+                }
+                mbar_expect_tx(bar0 + 40 + 8 * (kt & 1), uint32_t(T) * 128u);
+                tma_box_2d(base + uint32_t(kt & 1) * stage_bytes + a_bytes, &xmap, kt * kSearchKTile, 0, bar0 + 40 + 8 * (kt & 1));
+                x_started = kt;
+            }
+            // whatever was started lands before the block's shared memory is given up (long ago, unless the block gives up)
+            for (int j = x_started; j >= 0 && j > x_started - 2; --j) search_drain(bar0 + 40 + 8 * (j & 1), uint32_t((j >> 1) & 1));
+            for (int j = w_started; j >= 0 && j > w_started - 2; --j) search_drain(bar0 + 56 + 8 * (j & 1), uint32_t((j >> 1) & 1));
+        }
     } else {
         // this thread's part of a dW tile: row r of the block, 16 consecutive weights (2 pieces of 16 bytes)
         const int r = tid >> 2, quart = tid & 3;
@@ -228,46 +248,23 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
         const int slices_per_unit = p.L / kSearchKTile;
         const size_t s_at = size_t(blockIdx.z) * p.scale_stride + size_t(row_ok ? n : 0) * p.G;
         const __half *srow = p.S + s_at, *brow = p.qbias + s_at;
-        const int irow0 = int(blockIdx.z) * p.N + row0;   // W_int of the scale factors: one matrix of gridDim.z * N rows
         __half s_next = __float2half_rn(0.f), b_next = s_next;
         if (row_ok) s_next = __ldg(srow), b_next = __ldg(brow);
         float Sf = 0.f, qb = 0.f;
         __half Sh = s_next;
         int unit = 0, left = 0;   // slices left in the current scaling unit
 
-        // slices of X, W and W_int travel by tensor-map copies that one thread starts: W and W_int one slice ahead
-        // of their use, X as soon as the tensor cores have let go of the stage
-        int x_started = -1, w_started = -1;
-        if (tid == 0) {
-            mbar_expect_tx(bar0 + 56, kSearchWTile + kSearchITile);
-            tma_box_2d(base + a_bytes + x_bytes, &wmap, 0, row0, bar0 + 56);
-            tma_box_2d(base + a_bytes + x_bytes + kSearchWTile, &imap, 0, irow0, bar0 + 56);
-            w_started = 0;
-        }
-
-        for (int kt = 0; kt < ktiles && alive; ++kt) {
+        // The forming warps do not wait for one another: each waits for the stage (the MMAs that read it two slices ago) and for
+        // W, and publishes its part; a block-wide barrier per slice kept all of them in step, loads, arithmetic and stores one
+        // after the other.
+        for (int kt = 0; kt < ktiles; ++kt) {
             const int s = kt & 1;
             const uint32_t st_base = base + uint32_t(s) * stage_bytes;
-            // the MMAs that read this stage two slices ago must be complete before it is overwritten, and this slice
-            // of W must have landed (every thread takes the same decision: a wait that gives up must not split the
-            // block at a barrier)
             bool ok = kt < 2 || search_wait(bar0 + 8 * s, uint32_t(((kt >> 1) - 1) & 1), abort_flag, 1);
             ok = ok && search_wait(bar0 + 56 + 8 * s, uint32_t((kt >> 1) & 1), abort_flag, 5);
-            if (!formers_all(ok)) {
+            if (!__all_sync(0xffffffffu, ok)) {
                 alive = false;
                 break;
-            }
-            if (tid == 0) {
-                mbar_expect_tx(bar0 + 40 + 8 * s, uint32_t(T) * 128u);
-                tma_box_2d(st_base + a_bytes, &xmap, kt * kSearchKTile, 0, bar0 + 40 + 8 * s);
-                x_started = kt;
-                if (kt + 1 < ktiles) {   // the other stage's W was last read one slice ago, before that slice's barrier
-                    const uint32_t other = base + uint32_t(s ^ 1) * stage_bytes + a_bytes + x_bytes;
-                    mbar_expect_tx(bar0 + 56 + 8 * (s ^ 1), kSearchWTile + kSearchITile);
-                    tma_box_2d(other, &wmap, (kt + 1) * kSearchKTile, row0, bar0 + 56 + 8 * (s ^ 1));
-                    tma_box_2d(other + kSearchWTile, &imap, (kt + 1) * kSearchKTile, irow0, bar0 + 56 + 8 * (s ^ 1));
-                    w_started = kt + 1;
-                }
             }
 
             uint4 wcur0, wcur1, icur;
@@ -334,22 +331,18 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
                     }
                 });
             }
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the tiles are read by the tensor cores' proxy
-            named_barrier(1, kSearchThreads);                 // every forming thread's part of the stage is written and fenced
-            if (tid == 0) mbar_arrive(bar0 + 24 + 8 * s);     // the stage is full
+            // the tiles are read by the tensor cores' proxy, and W's slice is overwritten by the copies' proxy
+            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar0 + 24 + 8 * s);    // this warp's part of the stage is full
         }
-        if (tid == 0 && !alive) {   // giving up: the copies that were started still land in this block's shared memory
-            for (int j = x_started; j >= 0 && j > x_started - 2; --j) search_drain(bar0 + 40 + 8 * (j & 1), uint32_t((j >> 1) & 1));
-            for (int j = w_started; j >= 0 && j > w_started - 2; --j) search_drain(bar0 + 56 + 8 * (j & 1), uint32_t((j >> 1) & 1));
-        }
-
     }
 
     // ---- the accumulators are complete: every row's squared outputs ------------------------------------
     alive = __syncthreads_and((alive && search_wait(bar0 + 16, 0u, abort_flag, 2)) ? 1 : 0) != 0;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const int quarter = warp & 3, colpart = warp >> 2;   // a warp reads the 32 lanes of its quarter, every fourth piece of 16 columns
-    if (alive && warp < kSearchThreads / 32) {
+    if (alive && warp < kSearchFormers) {
         for (int c = 0; c < ncand; ++c) {
             float sum = 0.f;
             for (int ch = colpart; ch < T / 16; ch += 4) {
