@@ -134,7 +134,12 @@ cudaError_t launch_merge(const bcq_desc &d, const uint8_t *w_int, const uint16_t
                          uint8_t *codes, uint16_t *alpha, uint16_t *z, cudaStream_t st);
 cudaError_t launch_quantize_rtn(const uint16_t *W, int n_bits, double s_factor, const uint8_t *code_of_int /*[256]*/,
                                 const double *plane_weight /*[q]*/, uint16_t *S, uint16_t *qbias, uint8_t *w_int,
-                                const View &dst, cudaStream_t st, bool pack = true);   // pack = false: S, qbias, w_int only
+                                const View &dst, cudaStream_t st);
+// step 1 for the search: up to kStepOneScales scale factors in one pass over W (n_bits <= 6); per factor S, 4 W_int and
+// the residual S W_int + qbias - W in fp16
+constexpr int kStepOneScales = 8;
+cudaError_t launch_step_one(const uint16_t *W, int N, int K, int group, int n_bits, const double *s_factors, int scales, uint16_t *S,
+                            size_t scale_stride, uint16_t *qbias, uint8_t *offsets, uint16_t *resid, cudaStream_t st);
 cudaError_t launch_pack(const uint8_t *codes, const uint16_t *alpha_in, const uint16_t *z_in, const View &dst, cudaStream_t st);   // scales: into the tiles, or null
 cudaError_t launch_permute_planes(const View &src, const View &dst, cudaStream_t st);
 cudaError_t launch_permute_scales(const View &src, const View &dst, cudaStream_t st);
@@ -171,11 +176,11 @@ cudaError_t launch_mma_gemm(const bcq_desc &d, const bcq_plan &plan, const void 
 int record_cuda_error(cudaError_t e);   // text for bcq_last_cuda_error(); returns BCQ_ERR_CUDA
 
 // The search of section "Quantize Weight Twice" / "Re-explore Scale Factor": output errors of P candidates for
-// `scales` scale factors in one launch (step 1's outputs of the factors side by side: w_int [scales][N][K], S and
-// qbias `scale_stride` elements apart; err_rows [scales][P][N] per row, err [scales][P] summed in a fixed order),
+// `scales` scale factors in one launch (step 1's outputs of the factors side by side, see launch_step_one: offsets and
+// resid [scales][N][K], S `scale_stride` elements apart; err_rows [scales][P][N] per row, err [scales][P] summed in a fixed order),
 // and the first minimum of `count` errors laid out [.][P].
-cudaError_t launch_search_errors(const uint16_t *W, const uint8_t *w_int, const uint16_t *S, const uint16_t *qbias, size_t scale_stride,
-                                 const uint16_t *X, int N, int K, int group, int T, int n_bits, const float *lut_dev /*[P][64]*/, int P,
+cudaError_t launch_search_errors(const uint16_t *resid, const uint8_t *offsets, const uint16_t *S, size_t scale_stride, const uint16_t *X,
+                                 int N, int K, int group, int T, int n_bits, const float *lut_dev /*[P][64]*/, int P,
                                  int scales, float *err_rows, double *err, cudaStream_t st);
 cudaError_t launch_search_argmin(const double *err, int count, int P, int *best, cudaStream_t st);
 cudaError_t search_status_take(int *status);

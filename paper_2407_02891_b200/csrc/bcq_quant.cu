@@ -30,11 +30,11 @@ struct QuantTable {
     double s_factor;
 };
 
-__device__ __forceinline__ void range_to_scale(float lo, float hi, const QuantTable &tab, __half &s_h, __half &b_h)
+__device__ __forceinline__ void range_to_scale(float lo, float hi, double s_factor, double top, __half &s_h, __half &b_h)
 {
     if (lo == 0.f) lo = 0.f;   // a zero minimum is stored as +0
     const double range = double(hi) - double(lo);   // exact
-    s_h = __double2half(__ddiv_rn(__dmul_rn(tab.s_factor, range), tab.top));
+    s_h = __double2half(__ddiv_rn(__dmul_rn(s_factor, range), top));
     b_h = __float2half_rn(lo);                      // exact: lo is an fp16 value
 }
 
@@ -128,19 +128,78 @@ __device__ __forceinline__ uint32_t chunk_planes(const uint2 ints, const uint32_
     return spread;
 }
 
+// Range of a group of any length by one warp (NaN weights are ignored).
+__device__ __forceinline__ void warp_range(const __half *w, int L, float &lo, float &hi)
+{
+    const int lane = threadIdx.x & 31;
+    lo = __half2float(w[0]), hi = lo;
+#pragma unroll 4
+    for (int k = 8 * lane; k < L; k += 256) {   // L is a multiple of 32: whole 16-byte pieces
+        const uint4 raw = *reinterpret_cast<const uint4 *>(w + k);
+        const __half2 *h = reinterpret_cast<const __half2 *>(&raw);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float2 f = __half22float2(h[i]);
+            lo = fminf(lo, fminf(f.x, f.y));
+            hi = fmaxf(hi, fmaxf(f.x, f.y));
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    }
+}
+// the largest of a lane's 8 NR weights, NaN if there is one
+template <int NR>
+__device__ __forceinline__ __half lane_max(const uint4 (&raw)[NR])
+{
+    const __half2 *h = reinterpret_cast<const __half2 *>(raw);
+    __half2 hi2 = h[0];
+#pragma unroll
+    for (int i = 1; i < 4 * NR; ++i) hi2 = __hmax2_nan(hi2, h[i]);
+    return __hmax_nan(__low2half(hi2), __high2half(hi2));
+}
+// Range of a group that LANES neighbouring lanes hold, 8 NR weights each, in fp16 (exact).  A NaN weight is ignored by
+// (lo, hi_scale), but shows in hi: it makes the group go by the definition.
+template <int LANES, int NR>
+__device__ __forceinline__ void lanes_range(const uint4 (&raw)[NR], float &lo, float &hi, float &hi_scale)
+{
+    const __half2 *h = reinterpret_cast<const __half2 *>(raw);
+    __half2 lo2 = h[0];
+#pragma unroll
+    for (int i = 1; i < 4 * NR; ++i) lo2 = __hmin2(lo2, h[i]);
+    __half lo_h = __hmin(__low2half(lo2), __high2half(lo2)), hi_h = lane_max(raw);
+    for (int o = 1; o < LANES; o *= 2) {
+        const __half2 both = __halves2half2(lo_h, hi_h);
+        const uint32_t got = __shfl_xor_sync(0xffffffffu, *reinterpret_cast<const uint32_t *>(&both), o);
+        const __half2 other = *reinterpret_cast<const __half2 *>(&got);
+        lo_h = __hmin(lo_h, __low2half(other)), hi_h = __hmax_nan(hi_h, __high2half(other));
+    }
+    lo = __half2float(lo_h), hi = hi_scale = __half2float(hi_h);
+    if (__any_sync(0xffffffffu, hi != hi)) {
+        __half2 hi2 = h[0];
+#pragma unroll
+        for (int i = 1; i < 4 * NR; ++i) hi2 = __hmax2(hi2, h[i]);
+        hi_h = __hmax(__low2half(hi2), __high2half(hi2));
+        for (int o = 1; o < LANES; o *= 2) {
+            const uint32_t mine = __half_as_ushort(hi_h);
+            hi_h = __hmax(hi_h, __ushort_as_half(uint16_t(__shfl_xor_sync(0xffffffffu, mine, o))));
+        }
+        hi_scale = __half2float(hi_h);
+    }
+}
+
 // LANES: lanes per group, 4, 2 or 1 for groups of 128, 64 and 32 (one pass; jobs = (row unit, segment), segments
 // fastest); 0 for any other group length L: a block takes the row unit blockIdx.x, ranges first.
-// PACK = false (the search over scale factors wants the integers only): no planes, no fused scales.
-template <int FR, bool PACK, int LANES>
+template <int FR, int LANES>
 __global__ void __launch_bounds__(256, 3) rtn_kernel(const __half *__restrict__ W, const __grid_constant__ QuantTable tab, int L,
                                                   __half *S, __half *qbias, uint8_t *__restrict__ w_int, const View dst)
 {
     __shared__ uint32_t lut[256];
     const int lane = threadIdx.x & 31, j = lane >> 2, l = lane & 3, warp = threadIdx.x >> 5;
-    if (PACK) {
-        const uint32_t c = tab.code_of_int[threadIdx.x];
-        lut[threadIdx.x] = (c & 1u) | ((c & 2u) << 7) | ((c & 4u) << 14) | ((c & 8u) << 21);
-    }
+    const uint32_t code = tab.code_of_int[threadIdx.x];
+    lut[threadIdx.x] = (code & 1u) | ((code & 2u) << 7) | ((code & 4u) << 14) | ((code & 8u) << 21);
     const int N = dst.N, K = dst.K, G = K / L, q = dst.q;
     const int segs = (K + kSegment - 1) / kSegment;
 
@@ -149,30 +208,15 @@ __global__ void __launch_bounds__(256, 3) rtn_kernel(const __half *__restrict__ 
         for (int un = warp; un < rows * G; un += 8) {
             const int n = u * kUnitRows + un / G, g = un % G;
             const __half *w = W + size_t(n) * K + size_t(g) * L;
-            float lo = __half2float(w[0]), hi = lo;
-#pragma unroll 4
-            for (int k = 8 * lane; k < L; k += 256) {   // L is a multiple of 32: whole 16-byte pieces
-                const uint4 raw = *reinterpret_cast<const uint4 *>(w + k);
-                const __half2 *h = reinterpret_cast<const __half2 *>(&raw);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float2 f = __half22float2(h[i]);
-                    lo = fminf(lo, fminf(f.x, f.y));
-                    hi = fmaxf(hi, fmaxf(f.x, f.y));
-                }
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-                hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-            }
+            float lo, hi;
+            warp_range(w, L, lo, hi);
             __half s_h, b_h;
-            range_to_scale(lo, hi, tab, s_h, b_h);
+            range_to_scale(lo, hi, tab.s_factor, tab.top, s_h, b_h);
             if (lane == 0) {
                 S[size_t(n) * G + g] = s_h;
                 qbias[size_t(n) * G + g] = b_h;
             }
-            if (PACK && lane <= q) {
+            if (lane <= q) {
                 uint16_t *to = lane < q ? dst.alpha_elem(lane, n, g) : dst.z_elem(n, g);
                 *to = fused_scale(s_h, b_h, tab, q, lane);
             }
@@ -200,39 +244,16 @@ __global__ void __launch_bounds__(256, 3) rtn_kernel(const __half *__restrict__ 
         __half s_h, b_h;
         float lo, hi;
         if constexpr (LANES > 0) {
-            // the group's range in fp16 (exact); a NaN weight is ignored, but makes the group go by the definition
-            const __half2 *h = reinterpret_cast<const __half2 *>(raw);
-            __half2 lo2 = h[0], hi2 = h[0];
-#pragma unroll
-            for (int i = 1; i < 16; ++i) lo2 = __hmin2(lo2, h[i]), hi2 = __hmax2_nan(hi2, h[i]);
-            __half lo_h = __hmin(__low2half(lo2), __high2half(lo2)), hi_h = __hmax_nan(__low2half(hi2), __high2half(hi2));
-            for (int o = 1; o < LANES; o *= 2) {
-                const __half2 both = __halves2half2(lo_h, hi_h);
-                const uint32_t got = __shfl_xor_sync(0xffffffffu, *reinterpret_cast<const uint32_t *>(&both), o);
-                const __half2 other = *reinterpret_cast<const __half2 *>(&got);
-                lo_h = __hmin(lo_h, __low2half(other)), hi_h = __hmax_nan(hi_h, __high2half(other));
-            }
-            lo = __half2float(lo_h), hi = __half2float(hi_h);
-            float hi_scale = hi;
-            if (__any_sync(0xffffffffu, hi != hi)) {
-                hi2 = h[0];
-#pragma unroll
-                for (int i = 1; i < 16; ++i) hi2 = __hmax2(hi2, h[i]);
-                hi_h = __hmax(__low2half(hi2), __high2half(hi2));
-                for (int o = 1; o < LANES; o *= 2) {
-                    const uint32_t mine = __half_as_ushort(hi_h);
-                    hi_h = __hmax(hi_h, __ushort_as_half(uint16_t(__shfl_xor_sync(0xffffffffu, mine, o))));
-                }
-                hi_scale = __half2float(hi_h);
-            }
-            range_to_scale(lo, hi_scale, tab, s_h, b_h);
+            float hi_scale;
+            lanes_range<LANES>(raw, lo, hi, hi_scale);
+            range_to_scale(lo, hi_scale, tab.s_factor, tab.top, s_h, b_h);
             const int li = l & (LANES - 1);          // this lane inside its group
             const int g = seg * (4 / LANES) + l / LANES;
             if (in && li == 0) {
                 S[size_t(n) * G + g] = s_h;
                 qbias[size_t(n) * G + g] = b_h;
             }
-            if (PACK && in) {   // the group's lanes share out its q + 1 fused scales
+            if (in) {   // the group's lanes share out its q + 1 fused scales
                 constexpr int sub = 4 / LANES;
                 const int per = q + 1;
                 uint16_t *tile_scales = reinterpret_cast<uint16_t *>(dst.packed + dst.tile_base(seg >> 2, u) + size_t(q) * 512) +
@@ -246,12 +267,7 @@ __global__ void __launch_bounds__(256, 3) rtn_kernel(const __half *__restrict__ 
             const size_t unit = in ? size_t(n) * G + k / L : 0;
             s_h = S[unit], b_h = qbias[unit];
             lo = __half2float(b_h);
-            // (a NaN weight in a group that has other numbers shows up here, not in the range)
-            const __half2 *h = reinterpret_cast<const __half2 *>(raw);
-            __half2 hi2 = h[0];
-#pragma unroll
-            for (int i = 1; i < 16; ++i) hi2 = __hmax2_nan(hi2, h[i]);
-            hi = __half2float(__hmax_nan(__low2half(hi2), __high2half(hi2)));
+            hi = __half2float(lane_max(raw));   // (a NaN weight in a group that has other numbers shows up here, not in the range)
         }
         const IntDecision<FR> dec(s_h, b_h, lo, hi, tab.top);
         uint2 ints[4];
@@ -264,49 +280,53 @@ __global__ void __launch_bounds__(256, 3) rtn_kernel(const __half *__restrict__ 
 #pragma unroll
             for (int c = 0; c < 4; ++c) to[c] = ints[c];
         }
-        if (PACK) {
-            uint32_t p[4];   // byte i of p[c]: plane i's byte of chunk c
+        uint32_t p[4];   // byte i of p[c]: plane i's byte of chunk c
 #pragma unroll
-            for (int c = 0; c < 4; ++c) p[c] = chunk_planes(ints[c], lut);
-            unsigned char *at = out.at(dst, u, seg);
+        for (int c = 0; c < 4; ++c) p[c] = chunk_planes(ints[c], lut);
+        unsigned char *at = out.at(dst, u, seg);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                if (i < q) {
-                    const uint32_t ab = __byte_perm(p[0], p[1], 0x0040u + 0x11u * i), cd = __byte_perm(p[2], p[3], 0x0040u + 0x11u * i);
-                    const uint32_t w = out.word(__byte_perm(ab, cd, 0x5410u));
-                    if (in) *reinterpret_cast<uint32_t *>(at + i * stride) = w;
-                }
+        for (int i = 0; i < 4; ++i) {
+            if (i < q) {
+                const uint32_t ab = __byte_perm(p[0], p[1], 0x0040u + 0x11u * i), cd = __byte_perm(p[2], p[3], 0x0040u + 0x11u * i);
+                const uint32_t w = out.word(__byte_perm(ab, cd, 0x5410u));
+                if (in) *reinterpret_cast<uint32_t *>(at + i * stride) = w;
             }
         }
     }
     __threadfence();   // operands visible device-wide before the block counts as finished (products fetch them early)
 }
 
-template <int FR>
-static cudaError_t launch_rtn(const __half *w, const QuantTable &tab, __half *s, __half *b, uint8_t *w_int, const View &dst, cudaStream_t st,
-                              bool pack)
+// grid of the one-pass forms: as many blocks as the GPU holds, each walking many jobs (the set-up of a block and its
+// closing fence cost about as much as a job)
+static cudaError_t walk_grid(int N, int K, int per_sm, unsigned &grid)
 {
-    const int L = dst.group == 0 ? dst.K : dst.group;
-    const int lanes = (L == 128 || L == 64 || L == 32) ? L / 32 : 0;
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const long long blocks = lanes ? (segment_jobs(dst.N, dst.K) + 7) / 8 : (dst.N + kUnitRows - 1) / kUnitRows;
-    // one pass: as many blocks as the GPU holds, each walking many jobs (the set-up of a block and its closing fence
-    // cost about as much as a job); two passes: a block per row unit
-    const unsigned grid = unsigned(lanes ? (blocks < sms * 3LL ? blocks : sms * 3LL) : blocks);
-    const auto kernel = lanes == 4   ? (pack ? rtn_kernel<FR, true, 4> : rtn_kernel<FR, false, 4>)
-                        : lanes == 2 ? (pack ? rtn_kernel<FR, true, 2> : rtn_kernel<FR, false, 2>)
-                        : lanes == 1 ? (pack ? rtn_kernel<FR, true, 1> : rtn_kernel<FR, false, 1>)
-                                     : (pack ? rtn_kernel<FR, true, 0> : rtn_kernel<FR, false, 0>);
+    const long long blocks = (segment_jobs(N, K) + 7) / 8, most = static_cast<long long>(sms) * per_sm;
+    grid = unsigned(blocks < most ? blocks : most);
+    return cudaSuccess;
+}
+
+template <int FR>
+static cudaError_t launch_rtn(const __half *w, const QuantTable &tab, __half *s, __half *b, uint8_t *w_int, const View &dst, cudaStream_t st)
+{
+    const int L = dst.group == 0 ? dst.K : dst.group;
+    const int lanes = (L == 128 || L == 64 || L == 32) ? L / 32 : 0;
+    unsigned grid = unsigned((dst.N + kUnitRows - 1) / kUnitRows);   // two passes: a block per row unit
+    if (lanes) {
+        const cudaError_t e = walk_grid(dst.N, dst.K, 3, grid);
+        if (e != cudaSuccess) return e;
+    }
+    const auto kernel = lanes == 4 ? rtn_kernel<FR, 4> : lanes == 2 ? rtn_kernel<FR, 2> : lanes == 1 ? rtn_kernel<FR, 1> : rtn_kernel<FR, 0>;
     kernel<<<grid, 256, 0, st>>>(w, tab, L, s, b, w_int, dst);
     return cudaGetLastError();
 }
 
 cudaError_t launch_quantize_rtn(const uint16_t *W, int n_bits, double s_factor, const uint8_t *code_of_int /*[256]*/,
                                 const double *plane_weight /*[q]*/, uint16_t *S, uint16_t *qbias, uint8_t *w_int,
-                                const View &dst, cudaStream_t st, bool pack)
+                                const View &dst, cudaStream_t st)
 {
     QuantTable tab;
     for (int t = 0; t < 256; ++t) tab.code_of_int[t] = code_of_int[t];
@@ -317,7 +337,121 @@ cudaError_t launch_quantize_rtn(const uint16_t *W, int n_bits, double s_factor, 
     const __half *w = reinterpret_cast<const __half *>(W);
     __half *s = reinterpret_cast<__half *>(S), *b = reinterpret_cast<__half *>(qbias);
     // 16 fraction bits leave 7 integer bits in the mantissa
-    return n_bits <= 7 ? launch_rtn<16>(w, tab, s, b, w_int, dst, st, pack) : launch_rtn<15>(w, tab, s, b, w_int, dst, st, pack);
+    return n_bits <= 7 ? launch_rtn<16>(w, tab, s, b, w_int, dst, st) : launch_rtn<15>(w, tab, s, b, w_int, dst, st);
+}
+
+// ---- step 1 for the search: several scale factors in one pass over W -----------------------------------------------
+
+struct StepOneTable {
+    double top;
+    double s_factor[kStepOneScales];
+    int scales;
+};
+
+// Per scale factor f: S (fp16, [N][G], scale_stride elements apart), four times W_int ([N][K] bytes: the search uses it as
+// an offset into a table of words) and the residual of step 1, r = S W_int + qbias - W (fp32, rounded to fp16 once, [N][K]).
+// A warp takes eight rows of a 128-weight segment, four lanes per row; lane l holds chunks l, l + 4, l + 8, l + 12 of the
+// row's 16, so that every load and store covers whole 32-byte sectors (half sectors: 214 us against the 120 of eight
+// passes with 32 consecutive weights per lane, 4096 x 4096, eight factors).  UNIT: weights per scaling unit, 128 or 64;
+// 0: other multiples of 64, ranges first, a block per row unit (qbias keeps the minima).
+template <int UNIT>
+__global__ void __launch_bounds__(256, 2) step_one_kernel(const __half *__restrict__ W, const __grid_constant__ StepOneTable tab, int N, int K, int L,
+                                                          __half *S, size_t scale_stride, __half *qbias, uint8_t *__restrict__ offsets,
+                                                          __half *__restrict__ resid)
+{
+    const int lane = threadIdx.x & 31, j = lane >> 2, l = lane & 3, warp = threadIdx.x >> 5;
+    const int G = K / L, segs = (K + kSegment - 1) / kSegment;
+    constexpr bool kOnePass = UNIT != 0;
+    constexpr int kParts = UNIT == 128 ? 1 : 2, kChunks = 4 / kParts;   // a segment's parts with scales of their own
+    if constexpr (!kOnePass) {
+        const int u = blockIdx.x, rows = min(kUnitRows, N - u * kUnitRows);
+        for (int un = warp; un < rows * G; un += 8) {
+            const int n = u * kUnitRows + un / G, g = un % G;
+            float lo, hi;
+            warp_range(W + size_t(n) * K + size_t(g) * L, L, lo, hi);
+            if (lane < tab.scales) {
+                __half s_h, b_h;
+                range_to_scale(lo, hi, tab.s_factor[lane], tab.top, s_h, b_h);
+                S[lane * scale_stride + size_t(n) * G + g] = s_h;
+                if (lane == 0) qbias[size_t(n) * G + g] = b_h;
+            }
+        }
+        __syncthreads();
+    }
+    const int units = kOnePass ? (N + kUnitRows - 1) / kUnitRows : int(blockIdx.x) + 1;
+    SegmentWalk at_job(kOnePass ? (long long)blockIdx.x * 8 + warp : (long long)blockIdx.x * segs + warp,
+                       kOnePass ? (long long)gridDim.x * 8 : 8, segs);
+    const size_t plane = size_t(N) * K;
+    for (; at_job.u < units; at_job.next()) {
+        const int n = at_job.u * kUnitRows + j;
+#pragma unroll
+        for (int part = 0; part < kParts; ++part) {
+            const int k = at_job.seg * kSegment + 64 * part;   // (K is a multiple of 64)
+            const bool in = n < N && k < K;
+            const size_t at = in ? size_t(n) * K + k + 8 * l : 0, unit = in ? size_t(n) * G + k / L : 0;
+            uint4 raw[kChunks];
+#pragma unroll
+            for (int c = 0; c < kChunks; ++c) raw[c] = in ? *reinterpret_cast<const uint4 *>(W + at + 32 * c) : make_uint4(0u, 0u, 0u, 0u);
+            float lo, hi, hi_scale = 0.f;
+            __half b_h = __float2half_rn(0.f);
+            if constexpr (kOnePass) {
+                lanes_range<4>(raw, lo, hi, hi_scale);
+            } else {
+                b_h = qbias[unit];
+                lo = __half2float(b_h), hi = __half2float(lane_max(raw));
+            }
+#pragma unroll 1
+            for (int f = 0; f < tab.scales; ++f) {
+                __half s_h;
+                if constexpr (kOnePass) {
+                    range_to_scale(lo, hi_scale, tab.s_factor[f], tab.top, s_h, b_h);
+                    if (in && l == 0) S[f * scale_stride + unit] = s_h;
+                } else {
+                    s_h = S[f * scale_stride + unit];
+                }
+                const IntDecision<16> dec(s_h, b_h, lo, hi, tab.top);
+                const float sf = __half2float(s_h), bf = __half2float(b_h);
+#pragma unroll
+                for (int c = 0; c < kChunks; ++c) {
+                    const uint2 ints = piece_ints<16>(raw[c], dec, s_h, b_h, tab.top);
+                    const uint32_t word[4] = {raw[c].x, raw[c].y, raw[c].z, raw[c].w};
+                    uint32_t out[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float2 w2 = __half22float2(*reinterpret_cast<const __half2 *>(&word[i]));
+                        const uint32_t v4 = i < 2 ? ints.x : ints.y;   // an integer v as the fp32 number 2^23 + v, minus 2^23
+                        const float v0 = __uint_as_float(__byte_perm(v4, 0x4B000000u, 0x7650u + ((2 * i) & 3))) - 8388608.f;
+                        const float v1 = __uint_as_float(__byte_perm(v4, 0x4B000000u, 0x7650u + ((2 * i + 1) & 3))) - 8388608.f;
+                        const __half2 r = __floats2half2_rn(fmaf(sf, v0, bf - w2.x), fmaf(sf, v1, bf - w2.y));
+                        out[i] = *reinterpret_cast<const uint32_t *>(&r);
+                    }
+                    if (in) {
+                        *reinterpret_cast<uint2 *>(offsets + f * plane + at + 32 * c) = make_uint2(ints.x << 2, ints.y << 2);
+                        *reinterpret_cast<uint4 *>(resid + f * plane + at + 32 * c) = make_uint4(out[0], out[1], out[2], out[3]);
+                    }
+                }
+            }
+        }
+    }
+}
+
+cudaError_t launch_step_one(const uint16_t *W, int N, int K, int group, int n_bits, const double *s_factors, int scales, uint16_t *S,
+                            size_t scale_stride, uint16_t *qbias, uint8_t *offsets, uint16_t *resid, cudaStream_t st)
+{
+    StepOneTable tab;
+    tab.top = double((1u << n_bits) - 1u);
+    tab.scales = scales;
+    for (int f = 0; f < kStepOneScales; ++f) tab.s_factor[f] = f < scales ? s_factors[f] : 1.0;
+    const int L = group == 0 ? K : group;
+    unsigned grid = unsigned((N + kUnitRows - 1) / kUnitRows);
+    if (L == 128 || L == 64) {
+        const cudaError_t e = walk_grid(N, K, 2, grid);
+        if (e != cudaSuccess) return e;
+    }
+    const auto kernel = L == 128 ? step_one_kernel<128> : L == 64 ? step_one_kernel<64> : step_one_kernel<0>;
+    kernel<<<grid, 256, 0, st>>>(reinterpret_cast<const __half *>(W), tab, N, K, L, reinterpret_cast<__half *>(S), scale_stride,
+                                 reinterpret_cast<__half *>(qbias), offsets, reinterpret_cast<__half *>(resid));
+    return cudaGetLastError();
 }
 
 }  // namespace bcq

@@ -11,8 +11,8 @@
 // residual of step 1, fp32 and rounded to fp16 once; one fp16 fused multiply-add per pair of elements and candidate)
 // straight into shared memory in the 128-byte-swizzled K-major
 // operand layout, and a warp of its own issues tcgen05.mma (M = 128, N = T, K = 16, fp16 x fp16 -> fp32) into
-// one accumulator per candidate in tensor memory.  The slices of X (same layout), W and W_int arrive by tensor-map
-// copies that one thread starts: thousands of 16-byte loads per slice would hold the forming warps at the load
+// one accumulator per candidate in tensor memory.  The slices of X (same layout), r and W_int arrive by tensor-map
+// copies that one thread starts (r and W_int of all scale factors are written by one pass over W, launch_step_one): thousands of 16-byte loads per slice would hold the forming warps at the load
 // queue.  Two operand stages: the 16 forming warps publish a stage on its "full" mbarrier, the issuing warp hands it
 // back by tcgen05.commit on its "free" mbarrier, so the tensor cores work on one slice while the next is formed
 // (issuing 16 MMAs holds a thread for about a microsecond: a forming thread cannot do it).  At the end every row's
@@ -35,17 +35,14 @@ constexpr int kSearchKTile = 64;        // weights along K per stage: 128 bytes 
 constexpr int kSearchMaxCand = 4;       // candidates (accumulators) per block
 constexpr int kSearchATile = kSearchRows * kSearchKTile * 2;   // 16 KB
 constexpr int kSearchMaxT = 256;
-constexpr int kSearchWTile = kSearchRows * kSearchKTile * 2;   // a slice of W: 16 KB
+constexpr int kSearchWTile = kSearchRows * kSearchKTile * 2;   // a slice of the residuals: 16 KB
 constexpr int kSearchITile = kSearchRows * kSearchKTile;       // a slice of W_int: 8 KB
 constexpr int kSearchSpin = 1 << 22;
 
 static __device__ int g_search_status = 0;
 
 struct SearchParams {
-    const __half *W;        // [N][K]
-    const uint8_t *w_int;   // [N][K]
     const __half *S;        // [N][G] per scale factor, scale_stride elements apart
-    const __half *qbias;    // [N][G], likewise
     size_t scale_stride;
     const __half *X;        // [T][K]
     float *err_rows;        // [scale factor][P][N]
@@ -113,14 +110,14 @@ __device__ __forceinline__ void search_drain(uint32_t bar, uint32_t parity)
 }
 
 // grid (row tiles of 128, groups of cand_per_block candidates, scale factors); dynamic shared memory: 2 stages x
-// (cand_per_block x 16 KB of dW tiles | X's slice, T x 128 bytes rounded up to 1 KB | W's slice 16 KB | W_int's 8 KB),
+// (cand_per_block x 16 KB of dW tiles | X's slice, T x 128 bytes rounded up to 1 KB | the residual's slice 16 KB | W_int's 8 KB),
 // 1024-byte aligned.
 __global__ void __launch_bounds__(kSearchBlock, 1)
     search_error_kernel(const SearchParams p, const __grid_constant__ CUtensorMap xmap, const __grid_constant__ CUtensorMap wmap,
                         const __grid_constant__ CUtensorMap imap)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    // stage 0 free, stage 1 free, all done, stage 0/1 full, X of stage 0/1 landed, W and W_int of stage 0/1 landed
+    // stage 0 free, stage 1 free, all done, stage 0/1 full, X of stage 0/1 landed, residuals and W_int of stage 0/1 landed
     __shared__ __align__(8) unsigned long long bars[9];
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
@@ -135,7 +132,7 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
     const int T = p.T;
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     const uint32_t a_bytes = uint32_t(p.cand_per_block) * kSearchATile, x_bytes = (uint32_t(T) * 128u + 1023u) & ~1023u;
-    const uint32_t stage_bytes = a_bytes + x_bytes + kSearchWTile + kSearchITile;   // dW tiles | X | W | W_int
+    const uint32_t stage_bytes = a_bytes + x_bytes + kSearchWTile + kSearchITile;   // dW tiles | X | residuals | W_int
     const uint32_t bar0 = smem_u32(&bars[0]);
     volatile int *abort_flag = &abort_s;
 
@@ -197,15 +194,15 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
             __syncwarp();
         }
     } else if (warp == kSearchFormers + 1) {
-        // ---- the copying warp: W and W_int a slice ahead (their stage is read again when every forming warp has finished the
+        // ---- the copying warp: residuals and W_int a slice ahead (their stage is read again when every forming warp has finished the
         // slice before), X as soon as the tensor cores have let go of the stage ----
         if (lane == 0) {
-            const int row0 = blockIdx.x * kSearchRows, irow0 = int(blockIdx.z) * p.N + row0;   // W_int of the scale factors: one matrix of gridDim.z * N rows
+            const int irow0 = int(blockIdx.z) * p.N + int(blockIdx.x) * kSearchRows;   // the scale factors' matrices as one of gridDim.z * N rows
             int x_started = -1, w_started = -1;
             auto start_w = [&](int kt) {
                 const uint32_t to = base + uint32_t(kt & 1) * stage_bytes + a_bytes + x_bytes, bar = bar0 + 56 + 8 * (kt & 1);
                 mbar_expect_tx(bar, kSearchWTile + kSearchITile);
-                tma_box_2d(to, &wmap, kt * kSearchKTile, row0, bar);
+                tma_box_2d(to, &wmap, kt * kSearchKTile, irow0, bar);
                 tma_box_2d(to + kSearchWTile, &imap, kt * kSearchKTile, irow0, bar);
                 w_started = kt;
             };
@@ -233,8 +230,7 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
     } else {
         // this thread's part of a dW tile: row r of the block, 16 consecutive weights (2 pieces of 16 bytes)
         const int r = tid >> 2, quart = tid & 3;
-        const int row0 = blockIdx.x * kSearchRows;
-        const int n = row0 + r;
+        const int n = blockIdx.x * kSearchRows + r;
         const bool row_ok = n < p.N;
         const uint32_t a_row_off = uint32_t(r) * 128u;
         const uint32_t step_u32 = smem_u32(step_s);
@@ -244,13 +240,12 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
         const uint32_t w_off1 = a_bytes + x_bytes + uint32_t(r) * 128u + uint32_t(((2 * quart + 1) ^ (r & 7)) << 4);
         const uint32_t i_off = a_bytes + x_bytes + kSearchWTile + uint32_t(r) * 64u + uint32_t(quart << 4);
 
-        // scale and offset of (row, scaling unit): loaded one slice before the unit starts (rows beyond N keep 0)
+        // scale of (row, scaling unit): loaded one slice before the unit starts (rows beyond N keep 0)
         const int slices_per_unit = p.L / kSearchKTile;
         const size_t s_at = size_t(blockIdx.z) * p.scale_stride + size_t(row_ok ? n : 0) * p.G;
-        const __half *srow = p.S + s_at, *brow = p.qbias + s_at;
-        __half s_next = __float2half_rn(0.f), b_next = s_next;
-        if (row_ok) s_next = __ldg(srow), b_next = __ldg(brow);
-        float Sf = 0.f, qb = 0.f;
+        const __half *srow = p.S + s_at;
+        __half s_next = __float2half_rn(0.f);
+        if (row_ok) s_next = __ldg(srow);
         __half Sh = s_next;
         int unit = 0, left = 0;   // slices left in the current scaling unit
 
@@ -272,37 +267,28 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
             asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(wcur1.x), "=r"(wcur1.y), "=r"(wcur1.z), "=r"(wcur1.w) : "r"(st_base + w_off1));
             asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(icur.x), "=r"(icur.y), "=r"(icur.z), "=r"(icur.w) : "r"(st_base + i_off));
             if (left == 0) {
-                Sh = s_next, Sf = __half2float(s_next), qb = __half2float(b_next);
+                Sh = s_next;
                 left = slices_per_unit;
                 ++unit;
-                if (row_ok && unit < p.G) s_next = __ldg(srow + unit), b_next = __ldg(brow + unit);
+                if (row_ok && unit < p.G) s_next = __ldg(srow + unit);
             }
             --left;
 
-            // dW_p = S lut_p[v] + qbias - W = S (lut_p[v] - v) + r with r = S v + qbias - W, the residual of step 1.
-            // r: one fp32 fused multiply-add, rounded to fp16 once for all candidates.  Per candidate the step comes
+            // dW_p = S lut_p[v] + qbias - W = S (lut_p[v] - v) + r with r = S v + qbias - W, the residual of step 1, which comes
+            // ready (fp32, rounded to fp16 once for all candidates).  Per candidate the step comes
             // out of the lookup's byte as the fp16 number 1024 + byte (bit pattern 0x6400 | byte), minus 1152; one
             // fp16 fused multiply-add on a pair of weights then is the operand as it is stored (rounded once).
-            uint32_t resid[8];     // r of weights (2 j, 2 j + 1), fp16 pairs
-            uint32_t at[16];       // shared-memory address of the word of W_int's value
+            const uint32_t resid[8] = {wcur0.x, wcur0.y, wcur0.z, wcur0.w, wcur1.x, wcur1.y, wcur1.z, wcur1.w};   // of weights (2 j, 2 j + 1)
+            uint32_t at[16];       // shared-memory address of the word of W_int's value (the slice holds 4 W_int)
             {
-                const uint32_t w8[8] = {wcur0.x, wcur0.y, wcur0.z, wcur0.w, wcur1.x, wcur1.y, wcur1.z, wcur1.w};
                 const uint32_t i4[4] = {icur.x, icur.y, icur.z, icur.w};
-    #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const float2 f = __half22float2(*reinterpret_cast<const __half2 *>(&w8[j]));
-                    const float v0 = float((i4[j >> 1] >> (16 * (j & 1))) & 0xffu);
-                    const float v1 = float((i4[j >> 1] >> (16 * (j & 1) + 8)) & 0xffu);
-                    const __half2 h = __floats2half2_rn(fmaf(Sf, v0, qb - f.x), fmaf(Sf, v1, qb - f.y));
-                    resid[j] = *reinterpret_cast<const uint32_t *>(&h);
-                }
-    #pragma unroll
-                for (int j = 0; j < 16; ++j) at[j] = step_u32 + (((i4[j >> 2] >> (8 * (j & 3))) & 0xffu) << 2);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) at[j] = step_u32 + ((i4[j >> 2] >> (8 * (j & 3))) & 0xffu);
             }
             const __half2 S2 = __half2half2(Sh);
             const __half2 bias2 = __half2half2(__float2half_rn(-1152.f));
-            // (rows beyond N: W reads as zeros and the scale and offset are 0, so dW = 0 whatever W_int holds there --
-            // zeros, or the next scale factor's first rows)
+            // (rows beyond N hold zeros or the next scale factor's first rows: they are formed like the others and their
+            // outputs are not stored)
     #pragma unroll
             for (int i = 0; i < 2; ++i) {
                 uint32_t e[8];   // the words of weights 8 i .. 8 i + 7
@@ -414,7 +400,7 @@ int search_cand_per_block(int T)
     return c > kSearchMaxCand ? kSearchMaxCand : c;
 }
 
-// two stages of (dW tiles | X | W | W_int), each part a multiple of 1024 bytes, + room to align the first
+// two stages of (dW tiles | X | residuals | W_int), each part a multiple of 1024 bytes, + room to align the first
 size_t search_smem_bytes(int T)
 {
     const size_t x_bytes = (size_t(T) * 128 + 1023) / 1024 * 1024;
@@ -448,8 +434,8 @@ static cudaError_t search_tensor_map(CUtensorMap *map, const void *ptr, bool byt
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-cudaError_t launch_search_errors(const uint16_t *W, const uint8_t *w_int, const uint16_t *S, const uint16_t *qbias, size_t scale_stride,
-                                 const uint16_t *X, int N, int K, int group, int T, int n_bits, const float *lut_dev /*[P][64]*/, int P,
+cudaError_t launch_search_errors(const uint16_t *resid, const uint8_t *offsets, const uint16_t *S, size_t scale_stride, const uint16_t *X,
+                                 int N, int K, int group, int T, int n_bits, const float *lut_dev /*[P][64]*/, int P,
                                  int scales, float *err_rows /*[scales][P][N]*/, double *err /*[scales][P]*/, cudaStream_t st)
 {
     static bool configured[64] = {};
@@ -457,8 +443,7 @@ cudaError_t launch_search_errors(const uint16_t *W, const uint8_t *w_int, const 
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     SearchParams p = {};
-    p.W = reinterpret_cast<const __half *>(W), p.w_int = w_int;
-    p.S = reinterpret_cast<const __half *>(S), p.qbias = reinterpret_cast<const __half *>(qbias), p.scale_stride = scale_stride;
+    p.S = reinterpret_cast<const __half *>(S), p.scale_stride = scale_stride;
     p.X = reinterpret_cast<const __half *>(X), p.err_rows = err_rows;
     p.N = N, p.K = K, p.L = group == 0 ? K : group, p.G = K / p.L, p.P = P;
     p.lut_size = 1 << n_bits;
@@ -470,11 +455,11 @@ cudaError_t launch_search_errors(const uint16_t *W, const uint8_t *w_int, const 
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) configured[dev] = true;
     }
-    // the slices of W (the block's 128 rows; rows beyond N read as zeros) and W_int (the scale factors' matrices as one
-    // of scales * N rows)
+    // the slices of the residuals and of W_int (the scale factors' matrices as one of scales * N rows)
     CUtensorMap xmap, wmap, imap;
-    if ((e = search_tensor_map(&wmap, W, false, uint64_t(N), uint64_t(K), uint32_t(kSearchRows), true)) != cudaSuccess) return e;
-    if ((e = search_tensor_map(&imap, w_int, true, uint64_t(scales) * uint64_t(N), uint64_t(K), uint32_t(kSearchRows), false)) != cudaSuccess) return e;
+    const uint64_t rows = uint64_t(scales) * uint64_t(N);
+    if ((e = search_tensor_map(&wmap, resid, false, rows, uint64_t(K), uint32_t(kSearchRows), true)) != cudaSuccess) return e;
+    if ((e = search_tensor_map(&imap, offsets, true, rows, uint64_t(K), uint32_t(kSearchRows), false)) != cudaSuccess) return e;
     const unsigned row_tiles = unsigned((N + kSearchRows - 1) / kSearchRows);
     // the error is a sum over tokens: pieces of at most 256 tokens, one launch each, the later ones adding to err_rows
     // (pieces of about equal size, multiples of 16)
