@@ -871,28 +871,42 @@ __global__ void __launch_bounds__(kLutThreads, 1) lut_gemv_kernel(const typename
         }
     }
     if (split) {
-        // two passes over the warp's accumulator slots, 32 rows each: lane 8 g + j takes row j of slot 4 h + g
+        // The warp's accumulator slots, 32 rows at a time: lane 8 g + j takes row j of slot 4 h + g.  All the adds are on
+        // their way before the first answer is looked at (one after the other, every further 32 rows, and the second
+        // column, cost another round trip to L2 at the end of the launch).
+        constexpr int kHalves = kUnitsPerWarp / 4;
+        unsigned long long mine[kHalves][NB], before[kHalves][NB];
 #pragma unroll
-        for (int h = 0; h < kUnitsPerWarp / 4; ++h) {
+        for (int h = 0; h < kHalves; ++h) {
             const int a = 4 * h + g4;
             const int ul = kJ * (cw + kCons * (a / kJ)) + a % kJ;
-            if (ul < V) {
-                const size_t n = size_t(u0 + ul) * kUnitRows + jr;
-                const float v = g4 == 0 ? tot[4 * h] : (g4 == 1 ? tot[4 * h + 1] : (g4 == 2 ? tot[4 * h + 2] : tot[4 * h + 3]));
-                const unsigned long long mine = splitk_encode(v);
-                const unsigned long long before = atomicAdd(accum + n, mine);
-                if (splitk_arrivals(before) == p.k_splits - 1) {
-                    y[n] = finish ? lut_finish(splitk_decode_f32(before + mine, p.k_splits), p, n) : splitk_decode(before + mine, p.k_splits);
-                    accum[n] = 0;
+            const size_t n = size_t(u0 + ul) * kUnitRows + jr;
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                mine[h][b] = before[h][b] = 0;
+                if (ul < V) {
+                    float v;
+                    if constexpr (NB == 2)
+                        v = b == 0 ? (g4 == 0 ? tot[4 * h] : (g4 == 1 ? tot[4 * h + 1] : (g4 == 2 ? tot[4 * h + 2] : tot[4 * h + 3])))
+                                   : (g4 == 0 ? tot1[4 * h] : (g4 == 1 ? tot1[4 * h + 1] : (g4 == 2 ? tot1[4 * h + 2] : tot1[4 * h + 3])));
+                    else
+                        v = g4 == 0 ? tot[4 * h] : (g4 == 1 ? tot[4 * h + 1] : (g4 == 2 ? tot[4 * h + 2] : tot[4 * h + 3]));
+                    mine[h][b] = splitk_encode(v);
+                    before[h][b] = atomicAdd(accum + size_t(b) * p.N + n, mine[h][b]);
                 }
-                if constexpr (NB == 2) {
-                    const float v1 = g4 == 0 ? tot1[4 * h] : (g4 == 1 ? tot1[4 * h + 1] : (g4 == 2 ? tot1[4 * h + 2] : tot1[4 * h + 3]));
-                    const unsigned long long mine1 = splitk_encode(v1);
-                    const unsigned long long before1 = atomicAdd(accum + size_t(p.N) + n, mine1);
-                    if (splitk_arrivals(before1) == p.k_splits - 1) {
-                        y[Nop + n] = splitk_decode(before1 + mine1, p.k_splits);
-                        accum[size_t(p.N) + n] = 0;
-                    }
+            }
+        }
+#pragma unroll
+        for (int h = 0; h < kHalves; ++h) {
+            const int a = 4 * h + g4;
+            const int ul = kJ * (cw + kCons * (a / kJ)) + a % kJ;
+            const size_t n = size_t(u0 + ul) * kUnitRows + jr;
+#pragma unroll
+            for (int b = 0; b < NB; ++b) {
+                if (ul < V && splitk_arrivals(before[h][b]) == p.k_splits - 1) {
+                    const unsigned long long all = before[h][b] + mine[h][b];
+                    y[b * Nop + n] = finish ? lut_finish(splitk_decode_f32(all, p.k_splits), p, n) : splitk_decode(all, p.k_splits);
+                    accum[size_t(b) * p.N + n] = 0;
                 }
             }
         }

@@ -156,33 +156,29 @@ __global__ void __launch_bounds__(kMmaThreads, 1) mma_gemm_kernel(const __grid_c
     // outputs of one finished pair: rows m of both units, columns 2 t, 2 t + 1 (and 8 + those)
     auto emit = [&](int pair) {
         const int ua = u0 + 2 * pair;
+        unsigned long long before[NA], mine[NA];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            if (ua + h >= u1) continue;
-            const int n = (ua + h) * kUnitRows + m;
-            unsigned long long before[NA / 2], mine[NA / 2];
-#pragma unroll
-            for (int c = 0; c < NA / 2; ++c) {
-                const int b = 8 * (c >> 1) + 2 * t + (c & 1);
-                const float v = acc[4 * (c >> 1) + 2 * h + (c & 1)];
-                before[c] = 0, mine[c] = 0;
-                if (b < p.B) {
-                    if (p.split) {
-                        mine[c] = split_encode(v, p.fmt);
-                        before[c] = atomicAdd(p.accum + size_t(b) * p.N + n, mine[c]);
-                    } else {
-                        p.Y[size_t(b) * p.N + n] = __float2half_rn(v);
-                    }
+        for (int e = 0; e < NA; ++e) {   // all adds on their way before the first answer is looked at
+            const int h = (e >> 1) & 1, b = 8 * (e >> 2) + 2 * t + (e & 1);
+            const size_t at = size_t(b) * p.N + size_t(ua + h) * kUnitRows + m;
+            before[e] = mine[e] = 0;
+            if (ua + h < u1 && b < p.B) {
+                if (p.split) {
+                    mine[e] = split_encode(acc[e], p.fmt);
+                    before[e] = atomicAdd(p.accum + at, mine[e]);
+                } else {
+                    p.Y[at] = __float2half_rn(acc[e]);
                 }
             }
-            if (p.split) {
+        }
+        if (p.split) {
 #pragma unroll
-                for (int c = 0; c < NA / 2; ++c) {
-                    const int b = 8 * (c >> 1) + 2 * t + (c & 1);
-                    if (b < p.B && int(before[c] >> p.fmt.count_shift) == p.fmt.arrivals - 1) {
-                        p.Y[size_t(b) * p.N + n] = split_decode(before[c] + mine[c], p.fmt);
-                        p.accum[size_t(b) * p.N + n] = 0;
-                    }
+            for (int e = 0; e < NA; ++e) {
+                const int h = (e >> 1) & 1, b = 8 * (e >> 2) + 2 * t + (e & 1);
+                const size_t at = size_t(b) * p.N + size_t(ua + h) * kUnitRows + m;
+                if (ua + h < u1 && b < p.B && int(before[e] >> p.fmt.count_shift) == p.fmt.arrivals - 1) {
+                    p.Y[at] = split_decode(before[e] + mine[e], p.fmt);
+                    p.accum[at] = 0;
                 }
             }
         }
