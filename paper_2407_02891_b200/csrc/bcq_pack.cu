@@ -87,7 +87,7 @@ __device__ __forceinline__ uint32_t plane_word(const uint32_t (&z)[4], int i)
 
 // Q planes; SUB: scaling units per segment when the canonical scales (alpha, z) go into the tiles, else 0.
 template <int Q, int SUB>
-__global__ void __launch_bounds__(256) pack_kernel(const uint8_t *__restrict__ codes, const uint16_t *__restrict__ alpha,
+__global__ void __launch_bounds__(256, 4) pack_kernel(const uint8_t *__restrict__ codes, const uint16_t *__restrict__ alpha,
                                                    const uint16_t *__restrict__ z, const View dst)
 {
     const int lane = threadIdx.x & 31, j = lane >> 2, l = lane & 3;
@@ -165,7 +165,7 @@ cudaError_t launch_pack(const uint8_t *codes, const uint16_t *alpha_in, const ui
     if (e != cudaSuccess) return e;
     // as many blocks as the GPU holds, each walking many jobs: a block's closing fence costs more than a job
     const long long blocks = (segment_jobs(dst.N, dst.K) + 7) / 8;
-    const unsigned grid = unsigned(blocks < sms * 6LL ? blocks : sms * 6LL);
+    const unsigned grid = unsigned(blocks < sms * 4LL ? blocks : sms * 4LL);
     const int sub = alpha_in ? dst.subs() : 0;
     switch (dst.q) {
         case 1: launch_pack_q<1>(sub, grid, codes, alpha_in, z_in, dst, st); break;
