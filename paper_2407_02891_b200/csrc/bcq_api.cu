@@ -453,7 +453,7 @@ SearchLayout search_layout(const bcq_desc &d, int P, int n_scales, bool own_rows
     L.together = n_scales < kSearchScalesPerLaunch ? n_scales : kSearchScalesPerLaunch;
     L.w_int_each = size_t(d.N) * d.K, L.S_each = round_up(size_t(d.N) * G * 2, 256);
     size_t at = 0;
-    L.lut = at, at += round_up(size_t(P) * 64 * sizeof(float), 256);
+    L.lut = at, at += round_up(size_t(P) * 65 * sizeof(float), 256);   // tables, then the candidates' order
     L.w_int = at, at += round_up(L.w_int_each * L.together, 256);
     L.S = at, at += L.S_each * L.together;
     L.qbias = at, at += L.S_each;
@@ -903,11 +903,21 @@ int bcq_grid_search(const bcq_desc *desc, const uint16_t *W, const uint16_t *X, 
     for (int s = 0; s < n_scales; ++s)
         if (!(s_factors[s] > 0.0) || !(s_factors[s] < 1e30)) return BCQ_ERR_INVALID_ARG;
 
-    std::vector<float> lut(size_t(P) * 64);
+    std::vector<float> lut(size_t(P) * 65);
+    std::vector<int32_t> order;
+    std::vector<char> bytes(size_t(P), 1);   // candidates whose steps are all bytes come first
     for (int c = 0; c < P; ++c) {
-        rc = nearest_reachable(d.q, n_bits, partitions + size_t(c) * n_bits, lut.data() + size_t(c) * 64);
+        float *table = lut.data() + size_t(c) * 64;
+        rc = nearest_reachable(d.q, n_bits, partitions + size_t(c) * n_bits, table);
         if (rc != BCQ_OK) return rc;
+        for (int v = 0; v < (1 << n_bits); ++v)
+            if (!search_step_is_byte(int(table[v]) - v)) bytes[c] = 0;
     }
+    for (int want = 1; want >= 0; --want)
+        for (int c = 0; c < P; ++c)
+            if (bytes[c] == want) order.push_back(c);
+    memcpy(lut.data() + size_t(P) * 64, order.data(), size_t(P) * sizeof(int32_t));
+
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     unsigned char *base = static_cast<unsigned char *>(ws);
     float *lut_dev = reinterpret_cast<float *>(base + L.lut);
@@ -923,7 +933,8 @@ int bcq_grid_search(const bcq_desc *desc, const uint16_t *W, const uint16_t *X, 
         e = launch_step_one(W, d.N, d.K, d.group, n_bits, s_factors + s0, count, S, L.S_each / 2, qbias, w_int, resid, st);
         if (e != cudaSuccess) return cuda_fail(e);
         float *rows = err_rows ? err_rows + size_t(s0) * P * d.N : reinterpret_cast<float *>(base + L.err_rows);
-        e = launch_search_errors(resid, w_int, S, L.S_each / 2, X, d.N, d.K, d.group, T, n_bits, lut_dev, P, count, rows,
+        e = launch_search_errors(resid, w_int, S, L.S_each / 2, X, d.N, d.K, d.group, T, n_bits, lut_dev,
+                                 reinterpret_cast<const int *>(lut_dev) + size_t(P) * 64, P, count, rows,
                                  err_all + size_t(s0) * P, st);
         if (e != cudaSuccess) return cuda_fail(e);
     }

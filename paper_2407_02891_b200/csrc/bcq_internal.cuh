@@ -175,12 +175,21 @@ cudaError_t launch_mma_gemm(const bcq_desc &d, const bcq_plan &plan, const void 
 
 int record_cuda_error(cudaError_t e);   // text for bcq_last_cuda_error(); returns BCQ_ERR_CUDA
 
+// Can the step be given by the upper byte of its fp16 number (0 .. 8, even numbers to 16 and so on)?  A group of four
+// candidates all of whose steps can saves an addition per pair of weights and candidate (4096 x 4096, 5 bits into 3
+// planes, where 22 of 25 candidates can: the blocks take those first).
+__host__ __device__ inline bool search_step_is_byte(int step)
+{
+    int m = step < 0 ? -step : step;
+    while (m > 7 && m % 2 == 0) m /= 2;   // three significant bits
+    return m <= 7;
+}
 // The search of section "Quantize Weight Twice" / "Re-explore Scale Factor": output errors of P candidates for
 // `scales` scale factors in one launch (step 1's outputs of the factors side by side, see launch_step_one: offsets and
 // resid [scales][N][K], S `scale_stride` elements apart; err_rows [scales][P][N] per row, err [scales][P] summed in a fixed order),
 // and the first minimum of `count` errors laid out [.][P].
 cudaError_t launch_search_errors(const uint16_t *resid, const uint8_t *offsets, const uint16_t *S, size_t scale_stride, const uint16_t *X,
-                                 int N, int K, int group, int T, int n_bits, const float *lut_dev /*[P][64]*/, int P,
+                                 int N, int K, int group, int T, int n_bits, const float *lut_dev /*[P][64]*/, const int *order_dev /*[P]*/, int P,
                                  int scales, float *err_rows, double *err, cudaStream_t st);
 cudaError_t launch_search_argmin(const double *err, int count, int P, int *best, cudaStream_t st);
 cudaError_t search_status_take(int *status);

@@ -53,6 +53,7 @@ struct SearchParams {
     int tmem_cols;          // power of two >= 32 covering cand_per_block * T
     int lut_size;           // 2^n_bits <= 64
     const float *lut;       // [P][64]: lut[p][v] = the integer of BCchoice p nearest to v
+    const int *order;       // [P]: the candidates as the blocks take them (see search_step_is_byte)
 };
 
 __device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr)
@@ -121,8 +122,9 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
     __shared__ __align__(8) unsigned long long bars[9];
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
-    // per value v of W_int one word: byte c = 128 + lut_c[v] - v, the step from v to the nearest integer of the block's
-    // candidate c (between -63 and 63).  One lookup per operand element serves the four candidates.
+    // per value v of W_int one word: byte c stands for lut_c[v] - v, the step from v to the nearest integer of the block's
+    // candidate c (between -63 and 63): the upper byte of the step as fp16 if that is all of it for every step of the block,
+    // else 128 + step.  One lookup per operand element serves the four candidates.
     __shared__ uint32_t step_s[64];
     __shared__ float part[4][kSearchMaxCand][kSearchRows];
 
@@ -136,11 +138,19 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
     const uint32_t bar0 = smem_u32(&bars[0]);
     volatile int *abort_flag = &abort_s;
 
+    int cand[kSearchMaxCand];   // the block's candidates
+#pragma unroll
+    for (int c = 0; c < kSearchMaxCand; ++c) cand[c] = p.order[cand0 + min(c, ncand - 1)];
+    bool fits = true;
+    for (int v = tid; v < p.lut_size; v += kSearchBlock)
+        for (int c = 0; c < ncand; ++c) fits = fits && search_step_is_byte(int(p.lut[size_t(cand[c]) * 64 + v]) - v);
+    const bool byte_steps = __syncthreads_and(fits ? 1 : 0) != 0;
     for (int v = tid; v < p.lut_size; v += kSearchBlock) {
-        uint32_t word = 0x80808080u;   // candidates the block does not have: step 0
+        uint32_t word = byte_steps ? 0u : 0x80808080u;   // candidates the block does not have: step 0
         for (int c = 0; c < ncand; ++c) {
-            const int step = int(p.lut[size_t(cand0 + c) * 64 + v]) - v;   // the table holds integers
-            word = (word & ~(0xffu << (8 * c))) | (uint32_t(128 + step) << (8 * c));
+            const int step = int(p.lut[size_t(cand[c]) * 64 + v]) - v;   // the table holds integers
+            const uint32_t code = byte_steps ? uint32_t(__half_as_ushort(__int2half_rn(step))) >> 8 : uint32_t(128 + step);
+            word = (word & ~(0xffu << (8 * c))) | (code << (8 * c));
         }
         step_s[v] = word;
     }
@@ -233,7 +243,6 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
         const int n = blockIdx.x * kSearchRows + r;
         const bool row_ok = n < p.N;
         const uint32_t a_row_off = uint32_t(r) * 128u;
-        const uint32_t step_u32 = smem_u32(step_s);
         // W's slice lands with the 128-byte swizzle (16-byte piece ^ row & 7: a warp's loads then spread over
         // all banks), W_int's as it is
         const uint32_t w_off0 = a_bytes + x_bytes + uint32_t(r) * 128u + uint32_t(((2 * quart) ^ (r & 7)) << 4);
@@ -276,47 +285,54 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
 
             // dW_p = S lut_p[v] + qbias - W = S (lut_p[v] - v) + r with r = S v + qbias - W, the residual of step 1, which comes
             // ready (fp32, rounded to fp16 once for all candidates).  Per candidate the step comes
-            // out of the lookup's byte as the fp16 number 1024 + byte (bit pattern 0x6400 | byte), minus 1152; one
+            // out of the lookup's byte as the fp16 number itself, or as 1024 + byte (bit pattern 0x6400 | byte), minus 1152; one
             // fp16 fused multiply-add on a pair of weights then is the operand as it is stored (rounded once).
-            const uint32_t resid[8] = {wcur0.x, wcur0.y, wcur0.z, wcur0.w, wcur1.x, wcur1.y, wcur1.z, wcur1.w};   // of weights (2 j, 2 j + 1)
-            uint32_t at[16];       // shared-memory address of the word of W_int's value (the slice holds 4 W_int)
-            {
-                const uint32_t i4[4] = {icur.x, icur.y, icur.z, icur.w};
-#pragma unroll
-                for (int j = 0; j < 16; ++j) at[j] = step_u32 + ((i4[j >> 2] >> (8 * (j & 3))) & 0xffu);
-            }
-            const __half2 S2 = __half2half2(Sh);
-            const __half2 bias2 = __half2half2(__float2half_rn(-1152.f));
             // (rows beyond N hold zeros or the next scale factor's first rows: they are formed like the others and their
             // outputs are not stored)
-    #pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                uint32_t e[8];   // the words of weights 8 i .. 8 i + 7
-    #pragma unroll
-                for (int j = 0; j < 8; ++j) asm volatile("ld.shared.u32 %0, [%1];" : "=r"(e[j]) : "r"(at[8 * i + j]));
-                uint32_t pair01[4], pair23[4];   // bytes: candidates (0, 1) resp. (2, 3) of weights (2 j, 2 j + 1)
-    #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    pair01[j] = __byte_perm(e[2 * j], e[2 * j + 1], 0x5140u);
-                    pair23[j] = __byte_perm(e[2 * j], e[2 * j + 1], 0x7362u);
-                }
-                const int piece = 2 * quart + i;
-                const uint32_t dst = st_base + a_row_off + uint32_t((piece ^ (r & 7)) << 4);
-                static_for<0, kSearchMaxCand>([&](auto C) {
-                    constexpr int c = decltype(C)::value;
-                    if (c < ncand) {
-                        uint32_t packed[4];
-    #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            const uint32_t raw = __byte_perm(c < 2 ? pair01[j] : pair23[j], 0x64646464u, (c & 1) ? 0x4342u : 0x4140u);
-                            const __half2 step = __hadd2(*reinterpret_cast<const __half2 *>(&raw), bias2);
-                            const __half2 h = __hfma2(S2, step, *reinterpret_cast<const __half2 *>(&resid[4 * i + j]));
-                            packed[j] = *reinterpret_cast<const uint32_t *>(&h);
-                        }
-                        asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + uint32_t(c) * kSearchATile), "r"(packed[0]), "r"(packed[1]), "r"(packed[2]), "r"(packed[3]) : "memory");
+            const uint32_t resid[8] = {wcur0.x, wcur0.y, wcur0.z, wcur0.w, wcur1.x, wcur1.y, wcur1.z, wcur1.w};   // of weights (2 j, 2 j + 1)
+            const uint32_t i4[4] = {icur.x, icur.y, icur.z, icur.w};   // 4 W_int: byte offsets into the words
+            const __half2 S2 = __half2half2(Sh);
+            auto form = [&](auto BYTES) {
+                constexpr bool bytes = decltype(BYTES)::value;
+                const __half2 bias2 = __half2half2(__float2half_rn(-1152.f));
+#pragma unroll
+                for (int i = 0; i < 2; ++i) {
+                    uint32_t e[8];   // the words of weights 8 i .. 8 i + 7
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        e[j] = *reinterpret_cast<const uint32_t *>(reinterpret_cast<const unsigned char *>(step_s) +
+                                                                   __byte_perm(i4[2 * i + (j >> 2)], 0u, 0x4440u + (j & 3)));
+                    uint32_t pair01[4], pair23[4];   // bytes: candidates (0, 1) resp. (2, 3) of weights (2 j, 2 j + 1)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        pair01[j] = __byte_perm(e[2 * j], e[2 * j + 1], 0x5140u);
+                        pair23[j] = __byte_perm(e[2 * j], e[2 * j + 1], 0x7362u);
                     }
-                });
-            }
+                    const int piece = 2 * quart + i;
+                    const uint32_t dst = st_base + a_row_off + uint32_t((piece ^ (r & 7)) << 4);
+                    static_for<0, kSearchMaxCand>([&](auto C) {
+                        constexpr int c = decltype(C)::value;
+                        if (c < ncand) {
+                            uint32_t packed[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const uint32_t pair = c < 2 ? pair01[j] : pair23[j];
+                                const uint32_t raw = bytes ? __byte_perm(pair, 0u, (c & 1) ? 0x3424u : 0x1404u)
+                                                           : __byte_perm(pair, 0x64646464u, (c & 1) ? 0x4342u : 0x4140u);
+                                __half2 step = *reinterpret_cast<const __half2 *>(&raw);
+                                if constexpr (!bytes) step = __hadd2(step, bias2);
+                                const __half2 h = __hfma2(S2, step, *reinterpret_cast<const __half2 *>(&resid[4 * i + j]));
+                                packed[j] = *reinterpret_cast<const uint32_t *>(&h);
+                            }
+                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + uint32_t(c) * kSearchATile), "r"(packed[0]), "r"(packed[1]), "r"(packed[2]), "r"(packed[3]) : "memory");
+                        }
+                    });
+                }
+            };
+            if (byte_steps)
+                form(std::true_type{});
+            else
+                form(std::false_type{});
             // the tiles are read by the tensor cores' proxy, and W's slice is overwritten by the copies' proxy
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
@@ -355,7 +371,7 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
         const int row = blockIdx.x * kSearchRows + tid;
         if (row < p.N)
             for (int c = 0; c < ncand; ++c) {
-                float *out = p.err_rows + (size_t(blockIdx.z) * p.P + size_t(cand0 + c)) * p.N + row;
+                float *out = p.err_rows + (size_t(blockIdx.z) * p.P + size_t(p.order[cand0 + c])) * p.N + row;
                 const float sum = (part[0][c][tid] + part[1][c][tid]) + (part[2][c][tid] + part[3][c][tid]);
                 *out = p.accumulate ? *out + sum : sum;   // pieces of tokens run one after the other on the stream
             }
@@ -435,7 +451,7 @@ static cudaError_t search_tensor_map(CUtensorMap *map, const void *ptr, bool byt
 }
 
 cudaError_t launch_search_errors(const uint16_t *resid, const uint8_t *offsets, const uint16_t *S, size_t scale_stride, const uint16_t *X,
-                                 int N, int K, int group, int T, int n_bits, const float *lut_dev /*[P][64]*/, int P,
+                                 int N, int K, int group, int T, int n_bits, const float *lut_dev /*[P][64]*/, const int *order_dev /*[P]*/, int P,
                                  int scales, float *err_rows /*[scales][P][N]*/, double *err /*[scales][P]*/, cudaStream_t st)
 {
     static bool configured[64] = {};
@@ -447,7 +463,7 @@ cudaError_t launch_search_errors(const uint16_t *resid, const uint8_t *offsets, 
     p.X = reinterpret_cast<const __half *>(X), p.err_rows = err_rows;
     p.N = N, p.K = K, p.L = group == 0 ? K : group, p.G = K / p.L, p.P = P;
     p.lut_size = 1 << n_bits;
-    p.lut = lut_dev;
+    p.lut = lut_dev, p.order = order_dev;
     if (dev < 0 || dev >= 64 || !configured[dev]) {
         size_t most = 0;
         for (int t = 16; t <= kSearchMaxT; t += 16) most = search_smem_bytes(t) > most ? search_smem_bytes(t) : most;
