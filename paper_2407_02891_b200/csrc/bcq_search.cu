@@ -50,7 +50,8 @@ struct SearchParams {
     int T, P;               // T: tokens of this launch (a piece of at most 256 of the call's)
     int accumulate;         // add to err_rows instead of writing it (every piece but the first)
     int cand_per_block;     // 1..4, so that cand_per_block * T <= 512 columns of tensor memory
-    int tmem_cols;          // power of two >= 32 covering cand_per_block * T
+    int tmem_cols;          // power of two >= 32 covering cand_per_block accumulators of acc_cols columns
+    int tokens_first;       // the MMAs' roles (see search_tokens_first)
     int lut_size;           // 2^n_bits <= 64
     const float *lut;       // [P][64]: lut[p][v] = the integer of BCchoice p nearest to v
     const int *order;       // [P]: the candidates as the blocks take them (see search_step_is_byte)
@@ -173,8 +174,10 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem_base = tmem_base_s;
 
-    // instruction descriptor: fp32 accumulate, fp16 A and B, both K-major, N = T, M = 128
-    const uint32_t idesc = (1u << 4) | (uint32_t(T >> 3) << 17) | (uint32_t(kSearchRows >> 4) << 24);
+    // instruction descriptor: fp32 accumulate, fp16 A and B, both K-major, M = 128; N: tokens, or the rows of one or two
+    // candidates
+    const uint32_t idesc = (1u << 4) | (uint32_t(kSearchRows >> 4) << 24);
+    const uint32_t idesc_n = uint32_t((p.tokens_first ? kSearchRows : T) >> 3) << 17;
 
     const int ktiles = p.K / kSearchKTile;
     bool alive = true;
@@ -190,13 +193,22 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
             if (lane == 0) {
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint32_t st_base = base + uint32_t(s) * stage_bytes;
-                const uint64_t bdesc = smem_desc_sw128(st_base + a_bytes);
-                for (int c = 0; c < ncand; ++c) {
-                    const uint64_t adesc = smem_desc_sw128(st_base + uint32_t(c) * kSearchATile);
-                    const uint32_t d = tmem_base + uint32_t(c * T);
+                const uint64_t xdesc = smem_desc_sw128(st_base + a_bytes);
+                if (p.tokens_first) {
+                    for (int c = 0; c < ncand; c += 2) {   // two candidates' tiles lie one behind the other: 256 rows
+                        const uint64_t wdesc = smem_desc_sw128(st_base + uint32_t(c) * kSearchATile);
+                        const uint32_t both = idesc + (c + 1 < ncand ? 2u * idesc_n : idesc_n);
 #pragma unroll
-                    for (int j = 0; j < kSearchKTile / 16; ++j)   // 16 weights = 32 bytes further along the row
-                        umma_f16(d, adesc + uint64_t(2 * j), bdesc + uint64_t(2 * j), idesc, (kt > 0 || j > 0) ? 1u : 0u);
+                        for (int j = 0; j < kSearchKTile / 16; ++j)   // 16 weights = 32 bytes further along the row
+                            umma_f16(tmem_base + uint32_t(c * kSearchRows), xdesc + uint64_t(2 * j), wdesc + uint64_t(2 * j), both, (kt > 0 || j > 0) ? 1u : 0u);
+                    }
+                } else {
+                    for (int c = 0; c < ncand; ++c) {
+                        const uint64_t wdesc = smem_desc_sw128(st_base + uint32_t(c) * kSearchATile);
+#pragma unroll
+                        for (int j = 0; j < kSearchKTile / 16; ++j)
+                            umma_f16(tmem_base + uint32_t(c * T), wdesc + uint64_t(2 * j), xdesc + uint64_t(2 * j), idesc + idesc_n, (kt > 0 || j > 0) ? 1u : 0u);
+                    }
                 }
                 umma_commit(bar0 + 8 * s);
                 if (kt == ktiles - 1) umma_commit(bar0 + 16);
@@ -343,26 +355,52 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
     // ---- the accumulators are complete: every row's squared outputs ------------------------------------
     alive = __syncthreads_and((alive && search_wait(bar0 + 16, 0u, abort_flag, 2)) ? 1 : 0) != 0;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const int quarter = warp & 3, colpart = warp >> 2;   // a warp reads the 32 lanes of its quarter, every fourth piece of 16 columns
+    const int quarter = warp & 3, colpart = warp >> 2;   // a warp reads the 32 lanes of its quarter
+    auto read16 = [&](int col, float (&v)[16]) {
+        uint32_t w[16];
+        asm volatile(
+            "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+            : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7]), "=r"(w[8]),
+              "=r"(w[9]), "=r"(w[10]), "=r"(w[11]), "=r"(w[12]), "=r"(w[13]), "=r"(w[14]), "=r"(w[15])
+            : "r"(tmem_base + (uint32_t(quarter * 32) << 16) + uint32_t(col)));
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(w[j]);
+    };
     if (alive && warp < kSearchFormers) {
         for (int c = 0; c < ncand; ++c) {
-            float sum = 0.f;
-            for (int ch = colpart; ch < T / 16; ch += 4) {
-                uint32_t v[16];
-                const uint32_t taddr = tmem_base + (uint32_t(quarter * 32) << 16) + uint32_t(c * T + ch * 16);
-                asm volatile(
-                    "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-                    : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
-                      "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                    : "r"(taddr));
-                asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+            if (p.tokens_first) {
+                // lane = token, column = row: 32 rows per warp, squared, then added up over the 32 tokens; every exchange
+                // halves the rows a lane keeps, lane l ends up with row l (lanes beyond T hold whatever lay behind X)
+                float sq[32];
+                const bool token = quarter * 32 + lane < T;
 #pragma unroll
-                for (int j = 0; j < 16; ++j) {
-                    const float e = __uint_as_float(v[j]);
-                    sum = fmaf(e, e, sum);
+                for (int half = 0; half < 2; ++half) {
+                    float v[16];
+                    read16(c * kSearchRows + colpart * 32 + half * 16, v);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) sq[half * 16 + j] = token ? v[j] * v[j] : 0.f;
                 }
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    const bool up = (lane & o) != 0;
+#pragma unroll
+                    for (int j = 0; j < o; ++j) {
+                        const float send = up ? sq[j] : sq[j + o], keep = up ? sq[j + o] : sq[j];
+                        sq[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                    }
+                }
+                part[quarter][c][colpart * 32 + lane] = sq[0];
+            } else {   // lane = row, column = token: every fourth piece of 16 columns
+                float sum = 0.f;
+                for (int ch = colpart; ch < T / 16; ch += 4) {
+                    float v[16];
+                    read16(c * T + ch * 16, v);
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) sum = fmaf(v[j], v[j], sum);
+                }
+                part[colpart][c][quarter * 32 + lane] = sum;
             }
-            part[colpart][c][quarter * 32 + lane] = sum;
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -410,6 +448,10 @@ __global__ void search_argmin_kernel(const double *__restrict__ err, int count, 
     best[1] = at % P;
 }
 
+// Which operand the MMAs take as A.  Weights: 128 rows of one candidate against T tokens.  Tokens: up to 128 of them
+// against the rows of two candidates at once, which reads 12 instead of 16 KB of shared memory per 16 weights and pair of
+// candidates at 128 tokens (the pipe that bounds the kernel), but not less from 64 tokens down, and more than 128 do not fit.
+bool search_tokens_first(int T) { return T > 64 && T <= kSearchRows; }
 int search_cand_per_block(int T)
 {
     int c = 512 / T;
@@ -485,8 +527,9 @@ cudaError_t launch_search_errors(const uint16_t *resid, const uint8_t *offsets, 
         p.X = reinterpret_cast<const __half *>(X) + size_t(t0) * K;
         p.T = Tp, p.accumulate = t0 > 0 ? 1 : 0;
         p.cand_per_block = search_cand_per_block(Tp);
+        p.tokens_first = search_tokens_first(Tp) ? 1 : 0;
         int cols = 32;
-        while (cols < p.cand_per_block * Tp) cols *= 2;
+        while (cols < p.cand_per_block * (p.tokens_first ? kSearchRows : Tp)) cols *= 2;
         p.tmem_cols = cols;
         if ((e = search_tensor_map(&xmap, p.X, false, uint64_t(Tp), uint64_t(K), uint32_t(Tp), true)) != cudaSuccess) return e;   // all rows of the piece
         const unsigned groups = unsigned((P + p.cand_per_block - 1) / p.cand_per_block);

@@ -120,3 +120,14 @@ def test_grid_search_fullsize_sampled_rows(T):
     np.testing.assert_allclose(e, got.sum(axis=2), rtol=1e-5)
     si, pi = (int(v) for v in best.cpu().numpy())
     assert e[si, pi] == e.min()
+
+
+@pytest.mark.parametrize("N,K,T,q,group,n_bits,n_scales", [
+    (136, 256, 80, 2, 64, 4, 2),       # the fewest tokens that go first in the MMAs; groups of four and three candidates
+    (128, 320, 112, 3, 0, 5, 1),       # a last group of one candidate, groups with and without byte steps; K = 5 slices
+    (300, 192, 128, 3, 192, 4, 9),     # a last group of two; a scaling unit that is a multiple of 64 only; ragged rows
+    (128, 128, 64, 2, 128, 5, 1),      # the most tokens that go second
+    (128, 128, 144, 2, 128, 6, 1),     # likewise beyond 128; steps of up to 31
+])
+def test_grid_search_on_both_sides_of_its_rules(N, K, T, q, group, n_bits, n_scales):
+    _check(N, K, T, q, group, n_bits, n_scales, f"search2/{N}x{K}x{T}")
