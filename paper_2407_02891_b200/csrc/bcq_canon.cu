@@ -113,7 +113,8 @@ __global__ void __launch_bounds__(kCanonThreads, 2) canon_kernel(const __grid_co
     };
 
     for (int lo = w0; lo < w1; lo += p.phase_windows) {
-        const int nw = min(p.phase_windows, w1 - lo), end = 4 * (lo + nw);   // segments 4 lo .. end - 1
+        // segments 4 lo .. end - 1; the last window's segments beyond K have neither bits nor scales
+        const int nw = min(p.phase_windows, w1 - lo), end = min(4 * (lo + nw), (p.K + kCanonSegment - 1) / kCanonSegment);
         int seg = 4 * lo + warp;
         Words cur = fetch(seg, end), next = fetch(seg + kCanonWarps, end);   // on their way while x is staged
         if (lo > w0) __syncthreads();
@@ -152,13 +153,14 @@ __global__ void __launch_bounds__(kCanonThreads, 2) canon_kernel(const __grid_co
             if constexpr (MODE == kScaleWord) {
 #pragma unroll
                 for (int w = 0; w < 4; ++w) {
-                    const int g = min((seg * kCanonSegment + 32 * w) / p.L, p.G - 1);   // (words beyond K: x is zero there)
+                    const int k = seg * kCanonSegment + 32 * w, g = k / p.L;
+                    const bool in = k < p.K;   // words of the last segment beyond K: scales 0
 #pragma unroll
                     for (int i = 0; i < Q; ++i) {
-                        nz.v[i][w >> 1][2 * (w & 1)] = __ldg(al0 + i * splane + g) * 0x10001u;
-                        nz.v[i][w >> 1][2 * (w & 1) + 1] = __ldg(al1 + i * splane + g) * 0x10001u;
+                        nz.v[i][w >> 1][2 * (w & 1)] = in ? __ldg(al0 + i * splane + g) * 0x10001u : 0u;
+                        nz.v[i][w >> 1][2 * (w & 1) + 1] = in ? __ldg(al1 + i * splane + g) * 0x10001u : 0u;
                     }
-                    const float zz[2] = {h2f(__ldg(z0 + g)), h2f(__ldg(z1 + g))};
+                    const float zz[2] = {in ? h2f(__ldg(z0 + g)) : 0.f, in ? h2f(__ldg(z1 + g)) : 0.f};
                     const float2 xl = *reinterpret_cast<const float2 *>(xw + w * BR);
                     float2 xh = make_float2(0.f, 0.f);
                     if constexpr (WIDE) xh = *reinterpret_cast<const float2 *>(xw + w * BR + 8);

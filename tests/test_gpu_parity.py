@@ -201,6 +201,31 @@ def test_canonical_products(N, K, q, group, B):
     assert torch.equal(Y.view(torch.int16), Y2.view(torch.int16))
 
 
+@pytest.mark.parametrize("N,K,q,group,B", [(17, 640, 3, 128, 1), (17, 768, 2, 256, 9), (16, 1408, 1, 128, 4), (33, 1792, 4, 256, 2),
+                                           (17, 608, 3, 32, 1), (16, 992, 2, 0, 3)])
+def test_canonical_products_use_no_scale_but_a_rows_own(N, K, q, group, B):
+    """The last window of 512 weights is a partial one: NaN right behind the scales, and in one row's scales, shows in no
+    other row.  (alpha and z are views of larger buffers, whose tails are the NaN.)  Bound as above."""
+    p, codes, alpha, z, X = make_layer(f"own/{N}x{K}q{q}g{group}", N, K, q, group, B)
+    ref = oracle.forward_planes(p, alpha, z, X, group)
+    bad = N // 2
+    alpha, z = alpha.copy(), z.copy()
+    alpha[:, bad], z[bad] = np.nan, np.nan
+
+    def framed(a):
+        own = torch.full((a.size + 64,), float("nan"), dtype=torch.float16, device=DEV)
+        own[:a.size] = dev(a).reshape(-1)
+        return own[:a.size]
+
+    L = gpu_layer(N, K, q, group, bq.LAYOUT_CANONICAL, codes, alpha, z)
+    Y = torch.zeros((B, N), dtype=torch.float16, device=DEV)
+    bq.gemm_smallbatch(L.d, L.packed, framed(alpha), framed(z), dev(X), Y, B, None)
+    torch.cuda.synchronize()
+    y, others = Y.cpu().numpy(), np.arange(N) != bad
+    assert np.isnan(y[:, bad]).all()
+    assert rel_err(y[:, others], ref[:, others]) <= 2.0 ** -10
+
+
 @pytest.mark.parametrize("N,K,q,group", LUT_SHAPES)
 def test_gemv_lut_kernel_default_plan(N, K, q, group):
     p, codes, alpha, z, x = make_layer(f"lut/{N}x{K}", N, K, q, group)
