@@ -115,7 +115,8 @@ typedef struct bcq_desc {
  * 2 = tensor-core small-batch kernel (tiled layout, 2..16 columns per launch); kernels 1 and 2
  * are launched as row_blocks x k_splits thread blocks; k_splits > 1 needs the workspace.
  * Limits: at most 184 (kernel 1; 160 for q = 4 with two columns per launch) or 176 (kernel 2)
- * row units of 8 rows per block, at most 32 windows of 512 weights per K split.
+ * row units of 8 rows per block, at most 32 windows of 512 weights per K split.  Kernel 2 runs
+ * more than 31 K splits as 31.
  * reserved: 0.  The library's own tests set BCQ_PLAN_TEST_* bits there (kernel 1 only) to see a
  * bounded wait inside the kernel run out without anything faulting: SHORT_WAITS shortens the
  * limit of every wait to about a millisecond, WITHHOLD_TABLE makes the table builders keep a
@@ -144,8 +145,10 @@ int bcq_plan_default(const bcq_desc *desc, int B, int sm_count, bcq_plan *plan_o
 
 /* Bytes of workspace the plan needs (0 when k_splits == 1 and the generic kernel).  The
  * workspace holds the split-K partial sums and arrival counts (one 64-bit word per row and
- * column, in which the K splits' sums meet as fixed-point numbers in units of 2^-26; a split's
- * partial sum beyond +-131071, kernel 2 with few splits: beyond more, saturates).  It must be zero-filled once
+ * column, in which the K splits' sums meet as fixed-point numbers; kernel 1: in units of 2^-26, a
+ * split's partial sum beyond +-131071 saturates; kernel 2: in units of 2^-36, an output with a
+ * partial sum beyond +-4096 (up to 15 splits: +-32768), infinite or NaN is computed again as one
+ * sum).  It must be zero-filled once
  * (bcq_workspace_init) before its first use; every call leaves it zero where it has to be, so
  * it can be reused by later calls ON THE SAME STREAM.  Two products in flight at once
  * need two workspaces.  After a call that bcq_poll_status reported as timed out the counters

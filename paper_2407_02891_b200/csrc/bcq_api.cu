@@ -174,7 +174,8 @@ int plan_mma(const bcq_desc *d, int sm, int B, bcq_plan *out)
     const int rb_min = (U + kMmaMaxUnitsPerBlock - 1) / kMmaMaxUnitsPerBlock;
     const int at_once = mma_windows_at_once(d->q, d->group != 0, B);
     double best = -1.0;
-    for (int ks = (W + kMaxWindowsPerBlock - 1) / kMaxWindowsPerBlock; ks <= W && ks <= 64; ++ks) {
+    const int ks_min = (W + kMaxWindowsPerBlock - 1) / kMaxWindowsPerBlock;
+    for (int ks = ks_min; ks <= W && ks <= (ks_min > kMmaMaxSplits ? 64 : kMmaMaxSplits); ++ks) {
         for (int k = 0; k <= 16; ++k) {
             for (int j = 0; j <= (k == 1 ? 8 : 0); ++j) {
                 const int rb = k == 0 ? rb_min : (k * sm) / ks - j;
@@ -249,8 +250,8 @@ size_t plan_workspace(const bcq_desc *d, const bcq_plan *p, int B)
     if (p->k_splits <= 1) return 0;
     // kernel 1 runs one column per launch, or two when the scales live in the tiles
     if (p->kernel == 1) return split_workspace_bytes(d->N, (B >= 2 && pairs_ok(d)) ? 2 : 1);
-    // kernel 2: one 64-bit word per row and column; the size stays what callers have been told to provide, which is
-    // never less (k_splits >= 2)
+    // kernel 2: one 64-bit word per row and column; the size stays what callers have always been told to provide, which
+    // is never less (k_splits >= 2)
     if (p->kernel == 2) return size_t(16384) + size_t(p->k_splits) * B * d->N * sizeof(float);
     return 0;
 }

@@ -17,6 +17,7 @@ constexpr int kLutConsumersMax = 23; // consumer warps per block of the lookup-t
 constexpr int kLutUnitsPerWarp = 8;  // row units a consumer warp keeps accumulators for
 constexpr int kMaxWindowsPerBlock = 32; // windows one block may walk (bounds the planner's search)
 constexpr int kMmaWarps = 16;        // warps per block of the small-batch kernel
+constexpr int kMmaMaxSplits = 31;    // K splits the small-batch kernel runs (plans with more: as many)
 constexpr int kMmaMaxUnitsPerBlock = 176; // row units per block of it (the sums its pairs may have to keep in shared memory)
 constexpr int kMaxRowBlocks = 4096; // row blocks a plan may have
 

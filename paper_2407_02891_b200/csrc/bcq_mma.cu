@@ -19,8 +19,11 @@
 // one contiguous piece of memory) filled with bulk async copies.
 //
 // Split K: as in the batch-1 kernel, every output owns one 64-bit word of the workspace, to which a split adds its
-// fixed-point sum and an arrival; whoever completes a word stores y and clears the word.  The result does not depend on
-// the order of arrival.  All waits are bounded.
+// fixed-point sum and an arrival; whoever completes a word stores y and clears the word.  A sum that the word cannot hold
+// (infinite, not a number, very large) arrives as such, and whoever completes the word computes that output over all of K.
+// The result does not depend on the order of arrival.  (fp32 sums per split, added up by the last to arrive, take a fence and
+// two more round trips to L2, and leave the adding to the last block: 8192 x 8192, 8 columns, 4 splits 21.6 us against 19.5;
+// 2048 x 8192, 16 splits 14.6 against 6.9.)  All waits are bounded.
 //
 // Bound: dispatch of the tensor instruction (9 cycles) and of the half-rate instructions around it (2.5 per MMA: metadata,
 // signs of x, half-words of planes): 16 cycles per MMA and SM sub-partition at up to 8 columns, 13 at 16; then the fixed
@@ -37,6 +40,43 @@ constexpr int kMmaMaxSlotsPerWarp = 4;
 
 static_assert(8 * kMmaWarps * kMmaMaxSlotsPerWarp + 8 <= kMmaFixedBytes, "barrier area");
 
+// Split-K words: arrivals in the top bits, below them the arrivals whose sum is not in the word, then the sum of the
+// biased fixed-point partial sums.  The widths follow from the number of arrivals.  The unit is 2^-36, so that
+// even 31 roundings to it are at most 2^-32, a 128th of half a step of fp16's subnormal numbers; what is left is the
+// limit of a partial sum: 2^19 for 4 splits, 2^16 for 8, 2^15 for up to 15, 2^13 for 16, 2^12 for up to 31.
+constexpr int kMmaUnit = 36;
+struct SplitFormat {
+    int count_shift, odd_shift;
+    long long bias;
+    float limit;   // a power of two; sums whose magnitude is not below it are not in the word
+    int arrivals;
+};
+inline SplitFormat split_format(int arrivals)
+{
+    int cb = 1, lb = 0;
+    while ((1 << cb) <= arrivals) ++cb;
+    while ((1 << lb) < arrivals) ++lb;
+    SplitFormat f;
+    f.count_shift = 64 - cb, f.odd_shift = 64 - 2 * cb;
+    f.bias = 1ll << (f.odd_shift - lb - 1);
+    f.limit = float(double(f.bias) / double(1ll << kMmaUnit));
+    f.arrivals = arrivals;
+    return f;
+}
+__device__ __forceinline__ unsigned long long split_encode(float v, const SplitFormat &f)
+{
+    const bool in = fabsf(v) < f.limit;
+    const long long fixed = __float2ll_rn(in ? v * float(1ll << kMmaUnit) : 0.f);   // the product is exact
+    return (1ull << f.count_shift) + (in ? 0ull : 1ull << f.odd_shift) + (unsigned long long)(fixed + f.bias);
+}
+__device__ __forceinline__ bool split_complete(unsigned long long before, const SplitFormat &f) { return int(before >> f.count_shift) == f.arrivals - 1; }
+__device__ __forceinline__ bool split_odd(unsigned long long w, const SplitFormat &f) { return ((w & ((1ull << f.count_shift) - 1)) >> f.odd_shift) != 0; }
+__device__ __forceinline__ __half split_decode(unsigned long long w, const SplitFormat &f)
+{
+    const long long s = (long long)(w & ((1ull << f.odd_shift) - 1)) - (long long)f.arrivals * f.bias;
+    return __double2half(double(s) * (1.0 / double(1ll << kMmaUnit)));
+}
+
 __device__ int g_mma_status = 0;  // 0, or the code of the wait that ran out (sticky until taken)
 
 struct MmaParams {
@@ -49,6 +89,7 @@ struct MmaParams {
     int N, K, B;
     int u_base, u_rem, w_base, w_rem;   // even partitions: part r starts at r * base + min(r, rem), base + (r < rem) items
     int split;               // k_splits > 1
+    View view;               // the operand, for outputs that are computed on their own
     int phase_windows;       // windows whose x is staged at a time
     int depth;               // ring slots per warp
     int x_at, sum_at, ring_at;   // shared memory: constants and x; sums between phases; rings
@@ -57,6 +98,43 @@ struct MmaParams {
 };
 
 enum { kMmaWaitFull = 11, kMmaWaitDrain = 14 };
+
+// Outputs whose sum did not fit its split-K word, one after the other, by the whole warp: lane l has those of `which` (bit e:
+// row unit ua + (e / 2) % 2, column as in the kernel).  A lane takes every 32nd segment of 128 weights; signed sums of 128 in fp32 as in
+// the kernel, everything else in fp64.
+__device__ __noinline__ void mma_single_outputs(const MmaParams &p, int ua, unsigned which)
+{
+    const int lane = threadIdx.x & 31;
+    for (int e = 0; e < 8; ++e) {
+        for (unsigned lanes = __ballot_sync(0xffffffffu, (which >> e) & 1u); lanes; lanes &= lanes - 1) {
+            const int from = __ffs(lanes) - 1;   // its row and column
+            const int n = (ua + ((e >> 1) & 1)) * kUnitRows + (from >> 2), b = 8 * (e >> 2) + 2 * (from & 3) + (e & 1);
+            const __half *x = p.X + size_t(b) * p.K;
+            double sum = 0.0;
+            for (int seg = lane; seg < p.K / 128; seg += 32) {
+                const int g = p.view.group ? seg : 0;
+                float total = 0.f, plane[4] = {0.f, 0.f, 0.f, 0.f};
+                for (int kb = 16 * seg; kb < 16 * seg + 16; ++kb) {
+                    uint32_t bits[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) bits[i] = i < p.view.q ? *p.view.plane_byte(i, n, kb) : 0u;
+                    for (int j = 0; j < 8; ++j) {
+                        const float v = __half2float(x[8 * kb + j]);
+                        total += v;
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) plane[i] += (bits[i] >> j) & 1u ? v : -v;
+                    }
+                }
+                sum += double(__half2float(__ushort_as_half(*p.view.z_elem(n, g)))) * double(total);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (i < p.view.q) sum += double(__half2float(__ushort_as_half(*p.view.alpha_elem(i, n, g)))) * double(plane[i]);
+            }
+            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+            if (lane == 0) p.Y[size_t(b) * p.N + n] = __double2half(sum);
+        }
+    }
+}
 
 // Q planes; GROUPED: scales per (row, group of 128) inside the tiles, else per row in arrays;
 // WIDE: 9..16 columns (two MMAs per step), else at most 8.
@@ -154,6 +232,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) mma_gemm_kernel(const __grid_c
     for (int e = 0; e < NA; ++e) acc[e] = 0.f;
 
     // outputs of one finished pair: rows m of both units, columns 2 t, 2 t + 1 (and 8 + those)
+    int emitted = 0, emitted0 = 0;       // this warp's pairs so far (at most 7), and the first of them
+    unsigned long long single = 0;       // 8 bits per pair: this lane's outputs that are to be computed on their own
     auto emit = [&](int pair) {
         const int ua = u0 + 2 * pair;
         unsigned long long before[NA], mine[NA];
@@ -172,15 +252,21 @@ __global__ void __launch_bounds__(kMmaThreads, 1) mma_gemm_kernel(const __grid_c
             }
         }
         if (p.split) {
+            unsigned which = 0;
 #pragma unroll
             for (int e = 0; e < NA; ++e) {
                 const int h = (e >> 1) & 1, b = 8 * (e >> 2) + 2 * t + (e & 1);
                 const size_t at = size_t(b) * p.N + size_t(ua + h) * kUnitRows + m;
-                if (ua + h < u1 && b < p.B && int(before[e] >> p.fmt.count_shift) == p.fmt.arrivals - 1) {
-                    p.Y[at] = split_decode(before[e] + mine[e], p.fmt);
+                if (ua + h < u1 && b < p.B && split_complete(before[e], p.fmt)) {
+                    if (split_odd(before[e] + mine[e], p.fmt))
+                        which |= 1u << e;
+                    else
+                        p.Y[at] = split_decode(before[e] + mine[e], p.fmt);
                     p.accum[at] = 0;
                 }
             }
+            single |= (unsigned long long)which << (8 * emitted);
+            if (emitted++ == 0) emitted0 = pair;
         }
     };
 
@@ -363,6 +449,10 @@ __global__ void __launch_bounds__(kMmaThreads, 1) mma_gemm_kernel(const __grid_c
         }
     }
 
+    if (__any_sync(0xffffffffu, single != 0))
+        for (int i = 0; i < emitted; ++i)
+            mma_single_outputs(p, u0 + 2 * (emitted0 + i * (whole ? 1 : kMmaWarps)), unsigned(single >> (8 * i)) & 0xffu);
+
     // Gave up on a wait: copies this warp started may still be in flight.  See them land (bounded)
     // before the block's shared memory can be handed to another block.
     if (!alive && lane == 0) {
@@ -459,18 +549,20 @@ cudaError_t launch_mma_gemm(const bcq_desc &d, const bcq_plan &plan, const void 
     prm.K = d.K;
     prm.B = B;
     const int U = d.N / kUnitRows, W = d.K / kWindow;
+    const int splits = plan.k_splits < kMmaMaxSplits ? plan.k_splits : kMmaMaxSplits;
     prm.u_base = U / plan.row_blocks, prm.u_rem = U % plan.row_blocks;
-    prm.w_base = W / plan.k_splits, prm.w_rem = W % plan.k_splits;
+    prm.w_base = W / splits, prm.w_rem = W % splits;
     prm.ones = 0x3C003C00u;
-    prm.split = plan.k_splits > 1;
-    prm.fmt = split_format(plan.k_splits);
+    prm.split = splits > 1;
+    prm.fmt = split_format(splits);
+    prm.view = make_view(d, packed, alpha, z);
     const bool grouped = d.group != 0;
     const int windows = prm.w_base + (prm.w_rem ? 1 : 0), pairs = (prm.u_base + (prm.u_rem ? 1 : 0) + 1) / 2;
     const MmaLayout l = mma_layout(d.q, grouped, B, windows, pairs);
     if (l.phase_windows < 1 || l.depth < 1) return cudaErrorInvalidValue;
     prm.phase_windows = l.phase_windows, prm.depth = l.depth;
     prm.x_at = l.x_at, prm.sum_at = l.sum_at, prm.ring_at = l.ring_at;
-    const dim3 grid(plan.row_blocks, plan.k_splits);
+    const dim3 grid(plan.row_blocks, splits);
     switch (d.q) {
         case 1: return launch_mma_sel<1>(prm, grouped, grid, st);
         case 2: return launch_mma_sel<2>(prm, grouped, grid, st);

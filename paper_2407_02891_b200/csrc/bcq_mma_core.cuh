@@ -107,38 +107,4 @@ __device__ __forceinline__ float stage_word(const uint4 (&src)[4], unsigned char
     return sum;
 }
 
-// Split-K words (see bcq_lut_kernel.cuh): arrivals in the top bits, NaN arrivals below them, then the sum of the biased
-// fixed-point partial sums in units of 2^-26.  The widths follow from the number of arrivals, so that few splits leave
-// partial sums a wide range (4 splits: +-2^29; 64: +-131071).
-struct SplitFormat {
-    int count_shift, nan_shift;
-    long long bias;
-    float limit;
-    int arrivals;
-};
-inline SplitFormat split_format(int arrivals)
-{
-    int cb = 1, lb = 0;
-    while ((1 << cb) <= arrivals) ++cb;
-    while ((1 << lb) < arrivals) ++lb;
-    SplitFormat f;
-    f.count_shift = 64 - cb, f.nan_shift = 64 - 2 * cb;
-    f.bias = 1ll << (f.nan_shift - lb - 1);
-    f.limit = float(double(f.bias) / double(1 << 26) * (1.0 - 1.0 / 16777216.0));   // exact: below the bias by one fp32 step
-    f.arrivals = arrivals;
-    return f;
-}
-__device__ __forceinline__ unsigned long long split_encode(float v, const SplitFormat &f)
-{
-    const unsigned long long w = 1ull << f.count_shift;
-    if (v != v) return w + (1ull << f.nan_shift) + (unsigned long long)f.bias;
-    return w + (unsigned long long)(__float2ll_rn(fminf(fmaxf(v, -f.limit), f.limit) * 67108864.f) + f.bias);
-}
-__device__ __forceinline__ __half split_decode(unsigned long long w, const SplitFormat &f)
-{
-    if ((w & ((1ull << f.count_shift) - 1)) >> f.nan_shift) return __ushort_as_half((unsigned short)0x7fffu);   // a NaN partial sum
-    const long long s = (long long)(w & ((1ull << f.nan_shift) - 1)) - (long long)f.arrivals * f.bias;
-    return __double2half(double(s) * (1.0 / 67108864.0));
-}
-
 }  // namespace bcq

@@ -421,6 +421,62 @@ def test_small_batch_kernel_shares_pairs_and_phases(N, K, q, group, rb, ks, B):
         assert not ws.any()                # every word is cleared again
 
 
+def small_batch(N, K, q, group, rb, ks, codes, alpha, z, X):
+    B = X.shape[0]
+    L = gpu_layer(N, K, q, group, bq.LAYOUT_TILED, codes, alpha, z)
+    plan = bq.Plan(2, rb, ks, 0)
+    ws = bq.new_workspace(L.d, B, plan)
+    Y = torch.zeros((B, N), dtype=torch.float16, device=DEV)
+    for _ in range(2):
+        bq.gemm_smallbatch_plan(L.d, plan, L.packed, L.alpha, L.z, dev(X), Y, B, ws)
+    torch.cuda.synchronize()
+    bq.poll_status()
+    assert ws is None or not ws.any()
+    return Y.cpu().numpy()
+
+
+@pytest.mark.parametrize("N,W,q,ks,rb,B", [(40, 4, 3, 4, 2, 3), (16, 64, 1, 64, 1, 2), (24, 128, 2, 128, 2, 9), (16, 16, 4, 16, 1, 16)])
+def test_small_batch_splits_carry_any_partial_sum(N, W, q, ks, rb, B):
+    """Rows 0 .. 5: +inf and -inf in different splits; an infinity beside a large finite sum of the other sign; each alone; finite
+    sums of 3.8e9 that cancel to 30000; one of 32000 in a single split."""
+    K, group = 512 * W, 128
+    p, codes, alpha, z, X = make_layer(f"carry/{N}x{K}q{q}", N, K, q, group, B)
+    X = np.random.default_rng(W).integers(400, 600, X.shape).astype(np.float16)
+    X[:, -128:] = X[:, :128]
+    X[:, -1] -= np.float16(0.5)                       # 60000 times the difference: 30000
+    alpha, z = alpha.copy(), np.zeros_like(z)
+    alpha[:, :, :4], alpha[:, :, -4:] = 0, 0          # the first and the last window (different splits): offsets only
+    z[0, 0], z[0, -1] = np.inf, -np.inf
+    z[1, 0], z[1, -1] = np.inf, -60000.0
+    z[2, 0] = np.inf
+    z[3, -1] = -np.inf
+    z[4, 0], z[4, -1] = 60000.0, -60000.0
+    z[5, 1] = 0.5
+    with np.errstate(invalid="ignore"):
+        ref = oracle.forward_planes(p, alpha, z, X, group)
+    y = small_batch(N, K, q, group, rb, ks, codes, alpha, z, X).astype(np.float64)
+    assert np.isnan(ref[:, 0]).all() and np.isnan(y[:, 0]).all()
+    assert (y[:, 1] == np.inf).all() and (y[:, 2] == np.inf).all() and (y[:, 3] == -np.inf).all()
+    # row 4's sum is of the order of 3.8e9 until the last split is added: half an fp32 step, 2^7, per addition
+    assert np.abs(y[:, 4] - ref[:, 4]).max() <= 2.0 ** 7 * W
+    # fp32 sums, then one rounding to fp16
+    assert np.abs(y[:, 5:] - ref[:, 5:]).max() <= 2.0 ** -10 * np.abs(ref[:, 5:]).max()
+
+
+@pytest.mark.parametrize("N,W,q,ks,rb,B", [(48, 16, 3, 16, 3, 2), (16, 64, 1, 64, 1, 11), (128, 8, 2, 4, 2, 8)])
+def test_small_batch_splits_keep_small_sums(N, W, q, ks, rb, B):
+    """Outputs around 2^-16, below fp16's normal range: the one rounding to a multiple of 2^-24 is all that may be lost.  The
+    signed sums of 128 activations are exact in fp32 (multiples of 2^-24 below 1); K / 128 (q + 1) fused multiply-adds to sums
+    below 2^-13 lose at most 2^-38 each, the additions of the splits as much."""
+    K, group = 512 * W, 128
+    p, codes, alpha, z, X = make_layer(f"small/{N}x{K}q{q}", N, K, q, group, B)
+    X = (X * np.float16(2.0 ** -19)).astype(np.float16)
+    ref = oracle.forward_planes(p, alpha, z, X, group)
+    assert 0 < np.abs(ref).max() < 2.0 ** -14
+    y = small_batch(N, K, q, group, rb, ks, codes, alpha, z, X).astype(np.float64)
+    assert np.abs(y - ref).max() <= 2.0 ** -25 + (K / 128 * (q + 1) + ks) * 2.0 ** -38
+
+
 def test_small_batch_kernel_structured_inputs():
     """Unit activations pick out single weights: exact values, every (row, k) position distinguishable."""
     N, K, q, group, B = 64, 1024, 3, 128, 16
