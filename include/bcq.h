@@ -271,13 +271,15 @@ int bcq_multi_row_blocks(const bcq_desc *desc, const bcq_plan *plan, const int32
 /*
  * Y[b] = W X[b] for b < B, 1 <= B <= 16; X [B][K], Y [B][N] row-major fp16.  Every column is
  * an independent product (the paper defines batch 1 only; Eq. bcw + Eq. fuse_step3 per column).
- * B == 1 is bcq_gemv.  Tiled layout: by default B >= 5 (one scale per row: B >= 2) takes ONE
+ * B == 1 is bcq_gemv.  Tiled layout: by default B >= 5 (one scale per row: B >= 4) takes ONE
  * pass over the packed weights for all columns (plan kernel 2, the tensor-core kernel: the weight
- * bits select +x or -x, sums of 128 weights in fp32 are scaled by alpha in fp32) and B == 2 .. 4
- * run the lookup-table kernel on column pairs (plan kernel 1 with tables that hold two columns'
- * sums side by side: one pass over the weights and one 4-byte lookup per weight byte for both
- * columns of a pair; every column is bit-identical to bcq_gemv on it; bcq_plan_default tells
- * which).  The workspace depends on B: bcq_workspace_bytes(desc, B, plan).
+ * bits select +x or -x, sums of 128 weights in fp32 are scaled by alpha in fp32) and fewer columns
+ * run the lookup-table kernel (plan kernel 1): with groups of 128 on column pairs (tables that
+ * hold two columns' sums side by side: one pass over the weights and one 4-byte lookup per weight
+ * byte for both columns of a pair; every column is bit-identical to bcq_gemv_plan with that plan),
+ * with one scale per row column by column (B == 2, 3: plan and workspace are those of bcq_gemv,
+ * and every column is bit-identical to it); groups of 64 and 32 run it column by column for every
+ * B.  bcq_plan_default tells which.  The workspace depends on B: bcq_workspace_bytes(desc, B, plan).
  * Canonical layout: one pass over the planes for all columns (plan kernel 0, no workspace).
  * bcq_gemm_smallbatch_plan takes the decomposition from the caller; a plan with kernel 1 runs
  * the lookup-table kernel on two columns at a time when the scales live in the tiles (group

@@ -56,12 +56,13 @@ int device_sm_count(int *out)
     return BCQ_OK;
 }
 
-// From this many columns on the default plan is the tensor-core kernel.  With the scales in the tiles the lookup-table
-// kernel takes two columns per pass, and up to two such passes are the default: every column is then bit-identical to
-// bcq_gemv on it (8192 x 8192, q = 3: 10.9 us at two columns against 18.6; 19.6 and 21.2 at three and four against 18.7).
-// With one scale per row it takes a pass per column (8192 x 8192, two columns: q = 3 21.2 us against 19, q = 2 16.2
-// against 15.8; 4096 x 4096, q = 4: 14.5 against 7.7).
-constexpr int kSmallBatchMin = 2;
+// From this many columns on the default plan is the tensor-core kernel.  Below, every column is bit-identical to the batch-1
+// product of that column: that is kept although the tensor-core kernel is the faster one before these lines.  With the
+// scales in the tiles the lookup-table kernel takes two columns per pass (8192 x 8192, q = 3: 10.9 us at two columns against
+// 18.6; 19.6 and 21.2 at three and four against 18.7).  With one scale per row it takes a pass per column, with bcq_gemv's own
+// decomposition (8192 x 8192, two columns: q = 3 21.2 us against 18.4, q = 2 16.0 against 14.2; 4096 x 4096, q = 4: 14.4 against
+// 7.4; 36864 x 9216, q = 2: 44.8 against 46.9).
+constexpr int kSmallBatchMin = 4;
 constexpr int kSmallBatchMinPairs = 5;
 // column pairs and the tensor-core kernel exist for groups of 128 (and, the latter, one scale per row); groups of
 // 64 and 32 run the lookup-table kernel column by column

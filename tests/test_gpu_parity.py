@@ -421,6 +421,19 @@ def test_small_batch_kernel_shares_pairs_and_phases(N, K, q, group, rb, ks, B):
         assert not ws.any()                # every word is cleared again
 
 
+@pytest.mark.parametrize("N,K,q,B", [(1024, 4096, 3, 2), (776, 2560, 2, 3), (8, 512, 1, 2), (4096, 4096, 4, 3)])
+def test_two_and_three_columns_with_one_scale_per_row_are_single_products(N, K, q, B):
+    """By default: same bits as bcq_gemv on every column, with the workspace of a single product."""
+    p, codes, alpha, z, X = make_layer(f"rows23/{N}x{K}q{q}", N, K, q, 0, B)
+    L = gpu_layer(N, K, q, 0, bq.LAYOUT_TILED, codes, alpha, z)
+    ws = bq.new_workspace(L.d, 1)
+    Y = torch.zeros((B, N), dtype=torch.float16, device=DEV)
+    bq.gemm_smallbatch(L.d, L.packed, L.alpha, L.z, dev(X), Y, B, ws)
+    torch.cuda.synchronize()
+    for b in range(B):
+        assert np.array_equal(run_gemv(L, X[b]), Y[b].cpu().numpy().astype(np.float64))
+
+
 def small_batch(N, K, q, group, rb, ks, codes, alpha, z, X):
     B = X.shape[0]
     L = gpu_layer(N, K, q, group, bq.LAYOUT_TILED, codes, alpha, z)

@@ -156,6 +156,17 @@ def test_default_plan_is_valid_and_fills_the_gpu(N, K):
     assert bq.plan_default(bq.desc(N, K, 2, 0, bq.LAYOUT_TILED), 1, 148).kernel == 1     # one scale per row
 
 
+@pytest.mark.parametrize("N,K,q", [(8, 512, 1), (4096, 4096, 4), (7168, 28672, 3), (36864, 9216, 2)])
+def test_default_plan_of_two_and_three_columns_with_one_scale_per_row(N, K, q):
+    """They are single products one after the other: bcq_gemv's plan, and its workspace is enough."""
+    d = bq.desc(N, K, q, 0, bq.LAYOUT_TILED)
+    one = bq.plan_default(d, 1, 148)
+    for B in (2, 3):
+        p = bq.plan_default(d, B, 148)
+        assert (p.kernel, p.row_blocks, p.k_splits) == (1, one.row_blocks, one.k_splits)
+        assert bq.workspace_bytes(d, B, p) == bq.workspace_bytes(d, 1, one)
+
+
 def test_default_plans_are_remembered_consistently():
     """bcq_plan_default keeps its last plans in a small table: more shapes than the table holds, asked
     twice in different orders and for different batches, always give the same plan."""
