@@ -11,8 +11,10 @@
 // at a time.  Where 16-row blocks alone do not give every SM one, K is split over the blocks of a cluster, whose sums meet in
 // the first one's shared memory, in rank order.
 //
-// Scaling units: one per row or multiples of 128 are applied to the sum of a segment (of the whole row) in fp32; any other
-// multiple of 32 goes into the MMAs as the non-zeros, a value per word of 32 weights.
+// Scaling units: one per row or multiples of 128 are applied to the sum of a segment in fp32; any other multiple of 32 goes
+// into the MMAs as the non-zeros, a value per word of 32 weights.  Either way the MMAs add up one segment, the segments are
+// added in fp32: the tensor cores cut their running sum off at every step instead of rounding it (2048 x 11008, groups of 32,
+// 16 columns: 0.8 % of the outputs were not the correctly rounded ones with sums that ran along K, 0.1 % so).
 //
 // Bound: the MMAs (26 % of the tensor pipe, seven of eight columns unused at one column) and the latency of plane words and
 // scales, with two blocks on some SMs and one on the others.  4096 x 11008, q = 3, groups of 128: 18.4 us at one column (16.2
@@ -92,16 +94,15 @@ __global__ void __launch_bounds__(kCanonThreads, 2) canon_kernel(const __grid_co
     const unsigned char *xa0 = xs + (m < p.B ? m : 0) * kXColBytes + t * 16;        // columns beyond B: a staged one; not stored
     const unsigned char *xb0 = xs + (m + 8 < p.B ? m + 8 : 0) * kXColBytes + t * 16;
     float acc[NA], c[Q][4], ch[WIDE ? Q : 1][4];
-    float4 xtot = make_float4(0.f, 0.f, 0.f, 0.f);   // one scale per row: sums of x of columns 2t, 2t + 1, 8 + those
 #pragma unroll
     for (int e = 0; e < NA; ++e) acc[e] = 0.f;
+    [[maybe_unused]] uint16_t sc[2][Q + 1];   // the scales of rows m and m + 8 in unit g
+    auto fetch_scales = [&](int g) {
 #pragma unroll
-    for (int i = 0; i < Q; ++i)
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            c[i][e] = 0.f;
-            if constexpr (WIDE) ch[i][e] = 0.f;
-        }
+        for (int i = 0; i < Q; ++i) sc[0][i] = __ldg(al0 + i * splane + g), sc[1][i] = __ldg(al1 + i * splane + g);
+        sc[0][Q] = __ldg(z0 + g), sc[1][Q] = __ldg(z1 + g);
+    };
+    if constexpr (MODE == kScaleRow) fetch_scales(0);
     // acc += a * (lo4, hi4) for the rows of half h
     auto scaled = [&](int h, float a, const float (&lo4)[4], const float (&hi4)[4]) {
         acc[2 * h] = fmaf(a, lo4[2 * h], acc[2 * h]);
@@ -143,13 +144,7 @@ __global__ void __launch_bounds__(kCanonThreads, 2) canon_kernel(const __grid_co
                 bits[i][0] = __byte_perm(cur.a[i], cur.b[i], 0x5410u);
                 bits[i][1] = __byte_perm(cur.a[i], cur.b[i], 0x7632u);
             }
-            uint16_t sc[2][Q + 1];
-            if constexpr (MODE == kScaleSegment) {   // asked for now, used after the MMAs
-                const int g = seg * kCanonSegment / p.L;
-#pragma unroll
-                for (int i = 0; i < Q; ++i) sc[0][i] = __ldg(al0 + i * splane + g), sc[1][i] = __ldg(al1 + i * splane + g);
-                sc[0][Q] = __ldg(z0 + g), sc[1][Q] = __ldg(z1 + g);
-            }
+            if constexpr (MODE == kScaleSegment) fetch_scales(seg * kCanonSegment / p.L);   // asked for now, used after the MMAs
             if constexpr (MODE == kScaleWord) {
 #pragma unroll
                 for (int w = 0; w < 4; ++w) {
@@ -167,9 +162,11 @@ __global__ void __launch_bounds__(kCanonThreads, 2) canon_kernel(const __grid_co
                     const float l4[4] = {xl.x, xl.y, xl.x, xl.y}, h4[4] = {xh.x, xh.y, xh.x, xh.y};
                     scaled(0, zz[0], l4, h4), scaled(1, zz[1], l4, h4);
                 }
-                segment_sums<Q, WIDE, false>(bits, xa, xb, nz, c, ch);
+                segment_sums<Q, WIDE, true>(bits, xa, xb, nz, c, ch);
+#pragma unroll
+                for (int i = 0; i < Q; ++i) scaled(0, 1.f, c[i], ch[WIDE ? i : 0]), scaled(1, 1.f, c[i], ch[WIDE ? i : 0]);
             } else {
-                segment_sums<Q, WIDE, MODE == kScaleSegment>(bits, xa, xb, nz, c, ch);
+                segment_sums<Q, WIDE, true>(bits, xa, xb, nz, c, ch);
                 float4 xt = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                 for (int w = 0; w < 4; ++w) {
@@ -180,32 +177,16 @@ __global__ void __launch_bounds__(kCanonThreads, 2) canon_kernel(const __grid_co
                         xt.z += xh.x, xt.w += xh.y;
                     }
                 }
-                if constexpr (MODE == kScaleRow) {
-                    xtot.x += xt.x, xtot.y += xt.y, xtot.z += xt.z, xtot.w += xt.w;
-                } else {
-                    const float l4[4] = {xt.x, xt.y, xt.x, xt.y}, h4[4] = {xt.z, xt.w, xt.z, xt.w};
+                const float l4[4] = {xt.x, xt.y, xt.x, xt.y}, h4[4] = {xt.z, xt.w, xt.z, xt.w};
 #pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        scaled(h, h2f(sc[h][Q]), l4, h4);
+                for (int h = 0; h < 2; ++h) {
+                    scaled(h, h2f(sc[h][Q]), l4, h4);
 #pragma unroll
-                        for (int i = 0; i < Q; ++i) scaled(h, h2f(sc[h][i]), c[i], ch[WIDE ? i : 0]);
-                    }
+                    for (int i = 0; i < Q; ++i) scaled(h, h2f(sc[h][i]), c[i], ch[WIDE ? i : 0]);
                 }
             }
             cur = next, next = after;
         }
-    }
-    if constexpr (MODE == kScaleRow) {
-        const float l4[4] = {xtot.x, xtot.y, xtot.x, xtot.y}, h4[4] = {xtot.z, xtot.w, xtot.z, xtot.w};
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            scaled(h, h2f(__ldg(h ? z1 : z0)), l4, h4);
-#pragma unroll
-            for (int i = 0; i < Q; ++i) scaled(h, h2f(__ldg((h ? al1 : al0) + i * splane)), c[i], ch[WIDE ? i : 0]);
-        }
-    } else if constexpr (MODE == kScaleWord) {
-#pragma unroll
-        for (int i = 0; i < Q; ++i) scaled(0, 1.f, c[i], ch[WIDE ? i : 0]), scaled(1, 1.f, c[i], ch[WIDE ? i : 0]);
     }
 
     // ---- the warps' sums in order, then the cluster's ------------------------------------------------------------

@@ -226,6 +226,25 @@ def test_canonical_products_use_no_scale_but_a_rows_own(N, K, q, group, B):
     assert rel_err(y[:, others], ref[:, others]) <= 2.0 ** -10
 
 
+@pytest.mark.parametrize("group,B", [(32, 1), (32, 9), (0, 1), (0, 9), (256, 2)])
+def test_canonical_sums_do_not_drift_along_the_row(group, B):
+    """65536 positive terms, one block per 16 rows: whatever a running sum loses at each step adds up.  A segment of 128 is 8 steps
+    of the tensor cores, at most 2^-23 each; each warp then adds 64 of them, and the eight warps' sums are added, with roundings
+    of 2^-24: 2^-17.5 in all, beside the one rounding to fp16."""
+    N, K, L = 1200, 65536, group or 65536
+    rng = np.random.default_rng(group + B)
+    alpha = rng.uniform(0.25, 1.0, (1, N, K // L)).astype(np.float16)
+    X = np.exp2(rng.uniform(-17, -7, (B, K))).astype(np.float16)
+    ref = X.astype(np.float64).reshape(B, K // L, L).sum(axis=2) @ alpha[0].astype(np.float64).T
+    d = bq.desc(N, K, 1, group, bq.LAYOUT_CANONICAL)
+    Y = torch.zeros((B, N), dtype=torch.float16, device=DEV)
+    bq.gemm_smallbatch(d, torch.full((N * K // 8,), 255, dtype=torch.uint8, device=DEV), dev(alpha.reshape(-1)),
+                       torch.zeros(N * K // L, dtype=torch.float16, device=DEV), dev(X), Y, B, None)
+    torch.cuda.synchronize()
+    half_step = np.exp2(np.floor(np.log2(ref)) - 11)
+    assert (np.abs(Y.cpu().numpy().astype(np.float64) - ref) <= half_step + 2.0 ** -17.5 * ref).all()
+
+
 @pytest.mark.parametrize("N,K,q,group", LUT_SHAPES)
 def test_gemv_lut_kernel_default_plan(N, K, q, group):
     p, codes, alpha, z, x = make_layer(f"lut/{N}x{K}", N, K, q, group)
