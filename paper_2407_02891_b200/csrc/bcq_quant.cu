@@ -128,26 +128,74 @@ __device__ __forceinline__ uint32_t chunk_planes(const uint2 ints, const uint32_
     return spread;
 }
 
-// Range of a group of any length by one warp (NaN weights are ignored).
-__device__ __forceinline__ void warp_range(const __half *w, int L, float &lo, float &hi)
+// Ranges of M groups of any length by one warp, all M on their way together (NaN weights are ignored).  Lane 8 m + i (M = 1:
+// lane i) returns the range of group m; the other lanes' values are not used.
+template <int M>
+__device__ __forceinline__ void warp_ranges(const __half *const (&w)[M], int L, float &lo, float &hi)
 {
     const int lane = threadIdx.x & 31;
-    lo = __half2float(w[0]), hi = lo;
-#pragma unroll 4
-    for (int k = 8 * lane; k < L; k += 256) {   // L is a multiple of 32: whole 16-byte pieces
-        const uint4 raw = *reinterpret_cast<const uint4 *>(w + k);
-        const __half2 *h = reinterpret_cast<const __half2 *>(&raw);
+    __half2 lo2[M], hi2[M];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float2 f = __half22float2(h[i]);
-            lo = fminf(lo, fminf(f.x, f.y));
-            hi = fmaxf(hi, fmaxf(f.x, f.y));
+    for (int m = 0; m < M; ++m) lo2[m] = hi2[m] = __half2half2(w[m][0]);
+#pragma unroll (M == 1 ? 8 : 1)
+    for (int k = 8 * lane; k < L; k += 256) {   // L is a multiple of 32: whole 16-byte pieces
+        uint4 raw[M];
+#pragma unroll
+        for (int m = 0; m < M; ++m) raw[m] = *reinterpret_cast<const uint4 *>(w[m] + k);
+#pragma unroll
+        for (int m = 0; m < M; ++m) {
+            const __half2 *h = reinterpret_cast<const __half2 *>(&raw[m]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) lo2[m] = __hmin2(lo2[m], h[i]), hi2[m] = __hmax2(hi2[m], h[i]);
         }
     }
+    uint32_t both[M];   // (minimum, maximum) of a group, combined over the lanes
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+    for (int m = 0; m < M; ++m) {
+        __half a = __hmin(__low2half(lo2[m]), __high2half(lo2[m])), b = __hmax(__low2half(hi2[m]), __high2half(hi2[m]));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const __half2 mine = __halves2half2(a, b);
+            const uint32_t got = __shfl_xor_sync(0xffffffffu, *reinterpret_cast<const uint32_t *>(&mine), o);
+            const __half2 other = *reinterpret_cast<const __half2 *>(&got);
+            a = __hmin(a, __low2half(other)), b = __hmax(b, __high2half(other));
+        }
+        const __half2 r = __halves2half2(a, b);
+        both[m] = *reinterpret_cast<const uint32_t *>(&r);
+    }
+    uint32_t own = both[0];
+#pragma unroll
+    for (int m = 1; m < M; ++m) own = (lane >> 3) == m ? both[m] : own;
+    const __half2 r = *reinterpret_cast<const __half2 *>(&own);
+    lo = __low2float(r), hi = __high2float(r);
+}
+// The groups g0 .. g1 of a block's row unit u, a warp per group or, where groups are short, per four of them: their ranges
+// go to use(row, group, i, lo, hi), in the lanes i = 0 .. 7 of each.  (A warp per group of 96 has 12 lanes with weights and
+// waits for one load after the other: 4096 x 4032, 162 us, 72 so.)
+template <class Use>
+__device__ __forceinline__ void unit_ranges(const __half *W, int N, int K, int L, int u, int g0, int g1, const Use &use)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int rows = min(kUnitRows, N - u * kUnitRows), groups = g1 - g0 + 1, count = rows * groups;
+    auto row = [&](int i) { return u * kUnitRows + i / groups; };
+    auto group = [&](int i) { return g0 + i % groups; };
+    auto at = [&](int i) { return W + size_t(row(i)) * K + size_t(group(i)) * L; };
+    float lo, hi;
+    if (L > 512) {
+        for (int i = warp; i < count; i += 8) {
+            const __half *w[1] = {at(i)};
+            warp_ranges<1>(w, L, lo, hi);
+            if (lane < 8) use(row(i), group(i), lane, lo, hi);
+        }
+    } else {
+        for (int i = 4 * warp; i < count; i += 32) {
+            const __half *w[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) w[m] = at(min(i + m, count - 1));
+            warp_ranges<4>(w, L, lo, hi);
+            const int mine = i + (lane >> 3);
+            if (mine < count) use(row(mine), group(mine), lane & 7, lo, hi);
+        }
     }
 }
 // the largest of a lane's 8 NR weights, NaN if there is one
@@ -191,7 +239,8 @@ __device__ __forceinline__ void lanes_range(const uint4 (&raw)[NR], float &lo, f
 }
 
 // LANES: lanes per group, 4, 2 or 1 for groups of 128, 64 and 32 (one pass; jobs = (row unit, segment), segments
-// fastest); 0 for any other group length L: a block takes the row unit blockIdx.x, ranges first.
+// fastest); 0 for any other group length L: a block takes the row unit blockIdx.x, ranges first, and of its segments the
+// part blockIdx.y (groups that two parts share are done by both, with the same results).
 template <int FR, int LANES>
 __global__ void __launch_bounds__(256, 3) rtn_kernel(const __half *__restrict__ W, const __grid_constant__ QuantTable tab, int L,
                                                   __half *S, __half *qbias, uint8_t *__restrict__ w_int, const View dst)
@@ -203,41 +252,33 @@ __global__ void __launch_bounds__(256, 3) rtn_kernel(const __half *__restrict__ 
     const int N = dst.N, K = dst.K, G = K / L, q = dst.q;
     const int segs = (K + kSegment - 1) / kSegment;
 
-    if constexpr (LANES == 0) {   // ranges: a warp per (row, group) of the block's row unit
-        const int u = blockIdx.x, rows = min(kUnitRows, N - u * kUnitRows);
-        for (int un = warp; un < rows * G; un += 8) {
-            const int n = u * kUnitRows + un / G, g = un % G;
-            const __half *w = W + size_t(n) * K + size_t(g) * L;
-            float lo, hi;
-            warp_range(w, L, lo, hi);
-            __half s_h, b_h;
-            range_to_scale(lo, hi, tab.s_factor, tab.top, s_h, b_h);
-            if (lane == 0) {
-                S[size_t(n) * G + g] = s_h;
-                qbias[size_t(n) * G + g] = b_h;
-            }
-            if (lane <= q) {
-                uint16_t *to = lane < q ? dst.alpha_elem(lane, n, g) : dst.z_elem(n, g);
-                *to = fused_scale(s_h, b_h, tab, q, lane);
-            }
-        }
-    }
+    const int seg0 = LANES ? 0 : int((long long)segs * blockIdx.y / gridDim.y), seg1 = LANES ? segs : int((long long)segs * (blockIdx.y + 1) / gridDim.y);
+    if constexpr (LANES == 0)
+        unit_ranges(W, N, K, L, blockIdx.x, seg0 * kSegment / L, (min(seg1 * kSegment, K) - 1) / L,
+                    [&](int n, int g, int i, float lo, float hi) {
+                        __half s_h, b_h;
+                        range_to_scale(lo, hi, tab.s_factor, tab.top, s_h, b_h);
+                        if (i == 6) S[size_t(n) * G + g] = s_h;
+                        if (i == 7) qbias[size_t(n) * G + g] = b_h;
+                        if (i <= q) *(i < q ? dst.alpha_elem(i, n, g) : dst.z_elem(n, g)) = fused_scale(s_h, b_h, tab, q, i);
+                    });
     __syncthreads();
 
     const PlaneWriter out(dst);
     const size_t stride = dst.plane_stride();
     const int units = LANES ? (N + kUnitRows - 1) / kUnitRows : int(blockIdx.x) + 1;   // the walk ends there
-    SegmentWalk at_job(LANES ? (long long)blockIdx.x * 8 + warp : (long long)blockIdx.x * segs + warp, LANES ? (long long)gridDim.x * 8 : 8, segs);
+    SegmentWalk at_job(LANES ? (long long)blockIdx.x * 8 + warp : (long long)blockIdx.x * segs + seg0 + warp, LANES ? (long long)gridDim.x * 8 : 8, segs);
     uint4 raw[4];
+    auto more = [&](const SegmentWalk &w) { return w.u < units && (LANES || w.seg < seg1); };
     auto fetch = [&](const SegmentWalk &w) {
         const int n = w.u * kUnitRows + j, k = w.seg * kSegment + 32 * l;
-        const bool in = w.u < units && n < N && k < K;
+        const bool in = more(w) && n < N && k < K;
         const uint4 *src = reinterpret_cast<const uint4 *>(W + size_t(n) * K + k);
 #pragma unroll
         for (int c = 0; c < 4; ++c) raw[c] = in ? src[c] : make_uint4(0u, 0u, 0u, 0u);
     };
     fetch(at_job);
-    while (at_job.u < units) {
+    while (more(at_job)) {
         const int u = at_job.u, seg = at_job.seg;
         const int n = u * kUnitRows + j, k = seg * kSegment + 32 * l;
         const bool in = n < N && k < K;
@@ -296,16 +337,33 @@ __global__ void __launch_bounds__(256, 3) rtn_kernel(const __half *__restrict__ 
     __threadfence();   // operands visible device-wide before the block counts as finished (products fetch them early)
 }
 
+// Parts of a row unit's segments in the forms that take the ranges first: where there are fewer row units than the blocks the
+// GPU holds, as many parts as fill it (8 x 131072, one scale per row: 185 us with one block, 34 so; 128 x 28672: 50 and 25).
+// At most 16: with one scale per row every part ranges the whole rows.  At least a segment per warp.
+static cudaError_t unit_grid(int N, int K, int per_sm, dim3 &grid)
+{
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const int units = (N + kUnitRows - 1) / kUnitRows, segs = (K + kSegment - 1) / kSegment;
+    int parts = sms * per_sm / units;
+    parts = parts > 16 ? 16 : parts;
+    parts = parts > segs / 8 ? segs / 8 : parts;
+    grid = dim3(unsigned(units), unsigned(parts < 1 ? 1 : parts));
+    return cudaSuccess;
+}
+
 // grid of the one-pass forms: as many blocks as the GPU holds, each walking many jobs (the set-up of a block and its
 // closing fence cost about as much as a job)
-static cudaError_t walk_grid(int N, int K, int per_sm, unsigned &grid)
+static cudaError_t walk_grid(int N, int K, int per_sm, dim3 &grid)
 {
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     const long long blocks = (segment_jobs(N, K) + 7) / 8, most = static_cast<long long>(sms) * per_sm;
-    grid = unsigned(blocks < most ? blocks : most);
+    grid = dim3(unsigned(blocks < most ? blocks : most));
     return cudaSuccess;
 }
 
@@ -314,11 +372,9 @@ static cudaError_t launch_rtn(const __half *w, const QuantTable &tab, __half *s,
 {
     const int L = dst.group == 0 ? dst.K : dst.group;
     const int lanes = (L == 128 || L == 64 || L == 32) ? L / 32 : 0;
-    unsigned grid = unsigned((dst.N + kUnitRows - 1) / kUnitRows);   // two passes: a block per row unit
-    if (lanes) {
-        const cudaError_t e = walk_grid(dst.N, dst.K, 3, grid);
-        if (e != cudaSuccess) return e;
-    }
+    dim3 grid;
+    const cudaError_t e = lanes ? walk_grid(dst.N, dst.K, 3, grid) : unit_grid(dst.N, dst.K, 3, grid);
+    if (e != cudaSuccess) return e;
     const auto kernel = lanes == 4 ? rtn_kernel<FR, 4> : lanes == 2 ? rtn_kernel<FR, 2> : lanes == 1 ? rtn_kernel<FR, 1> : rtn_kernel<FR, 0>;
     kernel<<<grid, 256, 0, st>>>(w, tab, L, s, b, w_int, dst);
     return cudaGetLastError();
@@ -364,18 +420,14 @@ __global__ void __launch_bounds__(256, 2) step_one_kernel(const __half *__restri
     constexpr bool kOnePass = UNIT != 0;
     constexpr int kParts = UNIT == 128 ? 1 : 2, kChunks = 4 / kParts;   // a segment's parts with scales of their own
     if constexpr (!kOnePass) {
-        const int u = blockIdx.x, rows = min(kUnitRows, N - u * kUnitRows);
-        for (int un = warp; un < rows * G; un += 8) {
-            const int n = u * kUnitRows + un / G, g = un % G;
-            float lo, hi;
-            warp_range(W + size_t(n) * K + size_t(g) * L, L, lo, hi);
-            if (lane < tab.scales) {
+        unit_ranges(W, N, K, L, blockIdx.x, 0, G - 1, [&](int n, int g, int i, float lo, float hi) {
+            if (i < tab.scales) {
                 __half s_h, b_h;
-                range_to_scale(lo, hi, tab.s_factor[lane], tab.top, s_h, b_h);
-                S[lane * scale_stride + size_t(n) * G + g] = s_h;
-                if (lane == 0) qbias[size_t(n) * G + g] = b_h;
+                range_to_scale(lo, hi, tab.s_factor[i], tab.top, s_h, b_h);
+                S[i * scale_stride + size_t(n) * G + g] = s_h;
+                if (i == 0) qbias[size_t(n) * G + g] = b_h;
             }
-        }
+        });
         __syncthreads();
     }
     const int units = kOnePass ? (N + kUnitRows - 1) / kUnitRows : int(blockIdx.x) + 1;
@@ -443,7 +495,7 @@ cudaError_t launch_step_one(const uint16_t *W, int N, int K, int group, int n_bi
     tab.scales = scales;
     for (int f = 0; f < kStepOneScales; ++f) tab.s_factor[f] = f < scales ? s_factors[f] : 1.0;
     const int L = group == 0 ? K : group;
-    unsigned grid = unsigned((N + kUnitRows - 1) / kUnitRows);
+    dim3 grid(unsigned((N + kUnitRows - 1) / kUnitRows));
     if (L == 128 || L == 64) {
         const cudaError_t e = walk_grid(N, K, 2, grid);
         if (e != cudaSuccess) return e;

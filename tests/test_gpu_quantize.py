@@ -205,3 +205,21 @@ def test_quantize_rtn_weights_that_are_not_numbers(group):
     assert wi[3, 77] == 0
     e_wi[3, 77] = 0
     assert np.array_equal(wi, e_wi)
+
+
+@pytest.mark.parametrize("N,K,q,group", [
+    (5, 12288, 3, 0),        # a few long rows: a row unit's segments in twelve parts
+    (1, 131072, 2, 0),       # the most parts
+    (17, 4128, 3, 96),       # short groups, four at a time; parts that share groups, a last segment of 32 weights
+    (9, 4608, 2, 1536),      # long groups that parts share
+    (8, 2048, 4, 512),       # the longest group that goes four at a time; two parts
+    (3, 1056, 1, 352),       # one part, fewer groups than warps
+])
+def test_quantize_rtn_in_parts(N, K, q, group):
+    W = weights(f"q/parts/{N}x{K}", N, K)
+    W[N // 2, K // 2] = np.float16(6.0)                # a maximum that one part alone holds
+    b2p = [min(i, q - 1) for i in range(5)]
+    S, qb, wi, packed, a, z = run(W, q, group, bq.LAYOUT_CANONICAL, 5, b2p)
+    e_wi, e_S, e_qb, e_packed, e_a, e_z, _ = expected(W, q, group, bq.LAYOUT_CANONICAL, 5, b2p, 1.0)
+    assert same(S, e_S) and same(qb, e_qb) and same(wi, e_wi) and same(packed, e_packed)
+    assert same(a, e_a) and same(z, e_z)
