@@ -143,10 +143,15 @@ def _dev(*ts):
             raise ValueError("expected a CUDA tensor")
 
 
+# the raw handle of a device's current stream and the current device, without the stream object around them (2 us of a call's
+# 9.5); not part of torch's public interface, so a torch without them goes by the stream object
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_device = getattr(torch._C, "_cuda_getDevice", None)
+
+
 def _stream():
-    # the raw handle of the current stream, without the stream object around it (2 us of a call's 9.5)
-    if torch.cuda.is_initialized():
-        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    if _raw_stream is not None and _device is not None and torch.cuda.is_initialized():
+        return _raw_stream(_device())
     return torch.cuda.current_stream().cuda_stream
 
 

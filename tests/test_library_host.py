@@ -5,6 +5,7 @@ import os
 import re
 
 import pytest
+import torch
 
 from paper_2407_02891_b200 import binding as bq
 from paper_2407_02891_b200 import build as bq_build
@@ -246,3 +247,17 @@ def test_default_plans_are_valid_for_every_layout_variant():
         if p.kernel == 1:
             cols = 2 if (group == 128 and B >= 2) else 1
             assert need in (0, cols * N * 8)
+
+
+@pytest.mark.parametrize("missing", ["_raw_stream", "_device"])
+def test_stream_handle_without_torchs_private_functions(monkeypatch, missing):
+    class Stream:
+        cuda_stream = 4242
+
+    monkeypatch.setattr(torch.cuda, "is_initialized", lambda: True)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: Stream)
+    monkeypatch.setattr(bq, "_raw_stream", lambda device: 7 + device)
+    monkeypatch.setattr(bq, "_device", lambda: 1)
+    assert bq._stream() == 8
+    monkeypatch.setattr(bq, missing, None)
+    assert bq._stream() == 4242
