@@ -401,7 +401,9 @@ int bcq_gemv_noalloc(const bcq_desc *desc, const void *packed_dev, const uint16_
  *   err_dev [n_scales][P] fp64; err_rows_dev [n_scales][P][N] fp32 or NULL; best_dev [2] int32.
  *   workspace: bcq_grid_search_workspace(desc, T, n_bits, P, n_scales, err_rows_dev != NULL) bytes, 256-byte
  *   aligned; holds W_int, S and the residuals of step 1 (fp16) of up to 8 scale factors (searched together in one
- *   launch: 3 N K bytes each).  Asynchronous on `stream`.
+ *   launch) for as many rows at a time as fit: 3 K bytes per row and factor.  (All rows, if that is not more than a
+ *   GiB.  A smaller workspace is accepted down to about N K bytes per factor plus the size of a packed operand, and a
+ *   larger one is used up to all rows.)  Asynchronous on `stream`.
  */
 size_t bcq_grid_search_workspace(const bcq_desc *desc, int T, int n_bits, int P, int n_scales, int rows_given);
 int bcq_grid_search(const bcq_desc *desc, const uint16_t *W_dev, const uint16_t *X_dev, int T, int n_bits,

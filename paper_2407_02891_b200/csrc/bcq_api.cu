@@ -443,27 +443,60 @@ size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 // Scale factors are searched several per launch (a launch of 128-row blocks x groups of candidates alone leaves the
 // last wave of blocks partly empty): step 1's outputs of kSearchScalesPerLaunch factors sit side by side.
 constexpr int kSearchScalesPerLaunch = kStepOneScales;
+// Rows are searched as many at a time as fit (a launch's rows are independent of the others').  All of them take 3 bytes per weight
+// and factor, 5.6 GB for 28672 x 8192 with eight factors; what is enough, and what callers are told where it is more than a
+// GiB, is a byte per weight and factor, the scales and a packed operand, 2 GB (17.7 ms for all rows at a time, 17.1 - 17.5 so: step 1
+// is still in L2 when it is read).  Below a GiB all rows are the better choice: 4096 x 4096 1.08 ms against 1.21 in 0.14 GB, 512 x
+// 4096, 32 tokens, 0.13 against 0.42.
 struct SearchLayout {
-    size_t lut, w_int, resid, S, qbias, err, err_rows, total;
-    size_t w_int_each, S_each;   // bytes of one scale factor's W_int; of its S (and of qbias)
-    int together;                // scale factors per launch
+    size_t lut, err, err_rows, step;   // step: from here on step 1 of the rows of a launch
+    size_t total, accepted;            // what callers are told; what is enough
+    int together;                      // scale factors per launch
 };
+struct SearchStep {
+    size_t w_int, resid, S, qbias, end;   // from SearchLayout::step on
+    size_t S_each;                        // bytes of one scale factor's S (and of qbias)
+};
+SearchStep search_step(const bcq_desc &d, int together, int rows)
+{
+    SearchStep s;
+    const size_t each = size_t(rows) * d.K;
+    s.S_each = round_up(size_t(rows) * n_groups(d) * 2, 256);
+    s.w_int = 0;
+    s.resid = round_up(each * together, 256);
+    s.S = s.resid + round_up(2 * each * together, 256);
+    s.qbias = s.S + s.S_each * together;
+    s.end = s.qbias + s.S_each;
+    return s;
+}
+constexpr int kSearchRowTile = 128;   // rows of a block
+constexpr size_t kSearchAllRows = size_t(1) << 30;   // step 1 of all rows, as far as it is not more than this
 SearchLayout search_layout(const bcq_desc &d, int P, int n_scales, bool own_rows)
 {
     SearchLayout L;
-    const size_t G = size_t(n_groups(d));
-    L.together = n_scales < kSearchScalesPerLaunch ? n_scales : kSearchScalesPerLaunch;
-    L.w_int_each = size_t(d.N) * d.K, L.S_each = round_up(size_t(d.N) * G * 2, 256);
+    const size_t G = size_t(n_groups(d)), t = size_t(n_scales < kSearchScalesPerLaunch ? n_scales : kSearchScalesPerLaunch);
+    L.together = int(t);
     size_t at = 0;
     L.lut = at, at += round_up(size_t(P) * 65 * sizeof(float), 256);   // tables, then the candidates' order
-    L.w_int = at, at += round_up(L.w_int_each * L.together, 256);
-    L.S = at, at += L.S_each * L.together;
-    L.qbias = at, at += L.S_each;
-    L.resid = at, at += round_up(2 * L.w_int_each * L.together, 256);
     L.err = at, at += round_up(size_t(n_scales) * P * sizeof(double), 256);
-    L.err_rows = at, at += own_rows ? round_up(size_t(L.together) * P * d.N * sizeof(float), 256) : 0;
-    L.total = at;
+    L.err_rows = at, at += own_rows ? round_up(t * P * d.N * sizeof(float), 256) : 0;
+    L.step = at;
+    const size_t all = round_up(t * d.N * d.K, 256) + 2 * t * round_up(d.N * G * 2, 256) + round_up(size_t(d.q) * d.N * (d.K / 8), 256) +
+                       round_up(size_t(d.q) * d.N * G * 2, 256) + round_up(d.N * G * 2, 256);
+    const size_t whole = search_step(d, L.together, d.N).end, wanted = whole < kSearchAllRows ? whole : kSearchAllRows;
+    const size_t order = round_up(size_t(P) * 65 * sizeof(float), 256) - round_up(size_t(P) * 64 * sizeof(float), 256);
+    L.accepted = at + all - order;
+    L.total = L.accepted > at + wanted ? L.accepted : at + wanted;
     return L;
+}
+// the most rows whose step 1 fits `bytes`: all, a multiple of a block's, or, where not even a block's fit, fewer
+int search_rows_that_fit(const bcq_desc &d, int together, size_t bytes)
+{
+    if (search_step(d, together, d.N).end <= bytes) return d.N;
+    const int unit = search_step(d, together, kSearchRowTile).end <= bytes ? kSearchRowTile : 1;
+    int rows = 0;
+    while (rows + unit < d.N && search_step(d, together, rows + unit).end <= bytes) rows += unit;
+    return rows;
 }
 
 int check_search(const bcq_desc *desc, int T, int n_bits, int P, int n_scales)
@@ -901,7 +934,9 @@ int bcq_grid_search(const bcq_desc *desc, const uint16_t *W, const uint16_t *X, 
     if (!aligned(W, 16) || !aligned(X, 16) || !aligned(err, 8) || !aligned(err_rows, 4) || !aligned(best, 4) || !aligned(ws, 256))
         return BCQ_ERR_MISALIGNED;
     const SearchLayout L = search_layout(d, P, n_scales, err_rows == nullptr);
-    if (ws_bytes < L.total) return BCQ_ERR_WORKSPACE_TOO_SMALL;
+    if (ws_bytes < L.accepted) return BCQ_ERR_WORKSPACE_TOO_SMALL;
+    const int most = search_rows_that_fit(d, L.together, ws_bytes - L.step);
+    if (most < 1) return BCQ_ERR_WORKSPACE_TOO_SMALL;
     for (int s = 0; s < n_scales; ++s)
         if (!(s_factors[s] > 0.0) || !(s_factors[s] < 1e30)) return BCQ_ERR_INVALID_ARG;
 
@@ -923,21 +958,30 @@ int bcq_grid_search(const bcq_desc *desc, const uint16_t *W, const uint16_t *X, 
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     unsigned char *base = static_cast<unsigned char *>(ws);
     float *lut_dev = reinterpret_cast<float *>(base + L.lut);
-    uint8_t *w_int = base + L.w_int;
-    uint16_t *S = reinterpret_cast<uint16_t *>(base + L.S), *qbias = reinterpret_cast<uint16_t *>(base + L.qbias);
-    uint16_t *resid = reinterpret_cast<uint16_t *>(base + L.resid);
     double *err_all = reinterpret_cast<double *>(base + L.err);
+    int sms = 0;
+    rc = device_sm_count(&sms);
+    if (rc != BCQ_OK) return rc;
     // (pageable host memory: the copy has left the vector when the call returns)
     cudaError_t e = cudaMemcpyAsync(lut_dev, lut.data(), lut.size() * sizeof(float), cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) return cuda_fail(e);
     for (int s0 = 0; s0 < n_scales; s0 += L.together) {
         const int count = n_scales - s0 < L.together ? n_scales - s0 : L.together;
-        e = launch_step_one(W, d.N, d.K, d.group, n_bits, s_factors + s0, count, S, L.S_each / 2, qbias, w_int, resid, st);
-        if (e != cudaSuccess) return cuda_fail(e);
-        float *rows = err_rows ? err_rows + size_t(s0) * P * d.N : reinterpret_cast<float *>(base + L.err_rows);
-        e = launch_search_errors(resid, w_int, S, L.S_each / 2, X, d.N, d.K, d.group, T, n_bits, lut_dev,
-                                 reinterpret_cast<const int *>(lut_dev) + size_t(P) * 64, P, count, rows,
-                                 err_all + size_t(s0) * P, st);
+        float *row_errors = err_rows ? err_rows + size_t(s0) * P * d.N : reinterpret_cast<float *>(base + L.err_rows);
+        const int step_rows = search_rows_per_launch(d.N, most, T, P, count, sms);
+        for (int n0 = 0; n0 < d.N; n0 += step_rows) {
+            const int rows = d.N - n0 < step_rows ? d.N - n0 : step_rows;
+            const SearchStep at = search_step(d, count, rows);
+            uint8_t *w_int = base + L.step + at.w_int;
+            uint16_t *resid = reinterpret_cast<uint16_t *>(base + L.step + at.resid);
+            uint16_t *S = reinterpret_cast<uint16_t *>(base + L.step + at.S), *qbias = reinterpret_cast<uint16_t *>(base + L.step + at.qbias);
+            e = launch_step_one(W + size_t(n0) * d.K, rows, d.K, d.group, n_bits, s_factors + s0, count, S, at.S_each / 2, qbias, w_int, resid, st);
+            if (e != cudaSuccess) return cuda_fail(e);
+            e = launch_search_errors(resid, w_int, S, at.S_each / 2, X, rows, d.N, d.K, d.group, T, n_bits, lut_dev,
+                                     reinterpret_cast<const int *>(lut_dev) + size_t(P) * 64, P, count, row_errors + n0, st);
+            if (e != cudaSuccess) return cuda_fail(e);
+        }
+        e = launch_search_sums(row_errors, d.N, P * count, err_all + size_t(s0) * P, st);
         if (e != cudaSuccess) return cuda_fail(e);
     }
     e = launch_search_argmin(err_all, n_scales * P, P, best, st);

@@ -187,11 +187,13 @@ __host__ __device__ inline bool search_step_is_byte(int step)
 }
 // The search of section "Quantize Weight Twice" / "Re-explore Scale Factor": output errors of P candidates for
 // `scales` scale factors in one launch (step 1's outputs of the factors side by side, see launch_step_one: offsets and
-// resid [scales][N][K], S `scale_stride` elements apart; err_rows [scales][P][N] per row, err [scales][P] summed in a fixed order),
-// and the first minimum of `count` errors laid out [.][P].
+// resid [scales][rows][K], S `scale_stride` elements apart) and `rows` of N rows; err_rows [scales][P][N] from the first of the
+// rows on; their sums over all N rows, in a fixed order; and the first minimum of `count` errors laid out [.][P].
 cudaError_t launch_search_errors(const uint16_t *resid, const uint8_t *offsets, const uint16_t *S, size_t scale_stride, const uint16_t *X,
-                                 int N, int K, int group, int T, int n_bits, const float *lut_dev /*[P][64]*/, const int *order_dev /*[P]*/, int P,
-                                 int scales, float *err_rows, double *err, cudaStream_t st);
+                                 int rows, int N, int K, int group, int T, int n_bits, const float *lut_dev /*[P][64]*/, const int *order_dev /*[P]*/,
+                                 int P, int scales, float *err_rows, cudaStream_t st);
+cudaError_t launch_search_sums(const float *err_rows, int N, int candidates, double *err, cudaStream_t st);
+int search_rows_per_launch(int N, int most, int T, int P, int scales, int sms);
 cudaError_t launch_search_argmin(const double *err, int count, int P, int *best, cudaStream_t st);
 cudaError_t search_status_take(int *status);
 

@@ -46,7 +46,8 @@ struct SearchParams {
     size_t scale_stride;
     const __half *X;        // [T][K]
     float *err_rows;        // [scale factor][P][N]
-    int N, K, G, L;         // L = weights per scaling unit (K when one per row)
+    int N, K, G, L;         // N: rows of this launch; L = weights per scaling unit (K when one per row)
+    int err_stride;         // rows of err_rows per candidate
     int T, P;               // T: tokens of this launch (a piece of at most 256 of the call's)
     int accumulate;         // add to err_rows instead of writing it (every piece but the first)
     int cand_per_block;     // 1..4, so that cand_per_block * T <= 512 columns of tensor memory
@@ -409,7 +410,7 @@ __global__ void __launch_bounds__(kSearchBlock, 1)
         const int row = blockIdx.x * kSearchRows + tid;
         if (row < p.N)
             for (int c = 0; c < ncand; ++c) {
-                float *out = p.err_rows + (size_t(blockIdx.z) * p.P + size_t(p.order[cand0 + c])) * p.N + row;
+                float *out = p.err_rows + (size_t(blockIdx.z) * p.P + size_t(p.order[cand0 + c])) * p.err_stride + row;
                 const float sum = (part[0][c][tid] + part[1][c][tid]) + (part[2][c][tid] + part[3][c][tid]);
                 *out = p.accumulate ? *out + sum : sum;   // pieces of tokens run one after the other on the stream
             }
@@ -458,6 +459,31 @@ int search_cand_per_block(int T)
     return c > kSearchMaxCand ? kSearchMaxCand : c;
 }
 
+// tokens per launch: pieces of about equal size, multiples of 16
+static int search_piece(int T)
+{
+    const int pieces = (T + kSearchMaxT - 1) / kSearchMaxT;
+    return ((T + pieces - 1) / pieces + 15) / 16 * 16;
+}
+// Rows per launch where only `most` rows' step 1 (a multiple of 128) fit the workspace: the multiple of 128 with the fewest
+// rounds of blocks, one per SM (4096 x 4096, 25 candidates, 8 factors, 128 tokens: 32 tiles of rows are 1792 blocks, 13 rounds,
+// in launches of 10 tiles still 13, of 11 14).  Every launch also waits for its last blocks and for its step 1: a quarter of a round.
+int search_rows_per_launch(int N, int most, int T, int P, int scales, int sms)
+{
+    if (most >= N || most < kSearchRows) return most;
+    const int piece = search_piece(T), per_block = search_cand_per_block(piece);
+    const long long per_tile = (long long)((P + per_block - 1) / per_block) * scales;
+    const int tiles = (N + kSearchRows - 1) / kSearchRows;
+    auto rounds = [&](int t) { return (t * per_tile + sms - 1) / sms; };
+    long long best = -1;
+    int rows = kSearchRows;
+    for (int t = most / kSearchRows; t >= 1; --t) {
+        const long long quarters = 4 * (tiles / t * rounds(t) + (tiles % t ? rounds(tiles % t) : 0)) + (tiles + t - 1) / t;
+        if (best < 0 || quarters < best) best = quarters, rows = t * kSearchRows;
+    }
+    return rows;
+}
+
 // two stages of (dW tiles | X | residuals | W_int), each part a multiple of 1024 bytes, + room to align the first
 size_t search_smem_bytes(int T)
 {
@@ -493,8 +519,8 @@ static cudaError_t search_tensor_map(CUtensorMap *map, const void *ptr, bool byt
 }
 
 cudaError_t launch_search_errors(const uint16_t *resid, const uint8_t *offsets, const uint16_t *S, size_t scale_stride, const uint16_t *X,
-                                 int N, int K, int group, int T, int n_bits, const float *lut_dev /*[P][64]*/, const int *order_dev /*[P]*/, int P,
-                                 int scales, float *err_rows /*[scales][P][N]*/, double *err /*[scales][P]*/, cudaStream_t st)
+                                 int rows, int N, int K, int group, int T, int n_bits, const float *lut_dev /*[P][64]*/, const int *order_dev /*[P]*/,
+                                 int P, int scales, float *err_rows /*[scales][P][N], from the first of these rows on*/, cudaStream_t st)
 {
     static bool configured[64] = {};
     int dev = 0;
@@ -503,7 +529,7 @@ cudaError_t launch_search_errors(const uint16_t *resid, const uint8_t *offsets, 
     SearchParams p = {};
     p.S = reinterpret_cast<const __half *>(S), p.scale_stride = scale_stride;
     p.X = reinterpret_cast<const __half *>(X), p.err_rows = err_rows;
-    p.N = N, p.K = K, p.L = group == 0 ? K : group, p.G = K / p.L, p.P = P;
+    p.N = rows, p.err_stride = N, p.K = K, p.L = group == 0 ? K : group, p.G = K / p.L, p.P = P;
     p.lut_size = 1 << n_bits;
     p.lut = lut_dev, p.order = order_dev;
     if (dev < 0 || dev >= 64 || !configured[dev]) {
@@ -513,15 +539,14 @@ cudaError_t launch_search_errors(const uint16_t *resid, const uint8_t *offsets, 
         if (e != cudaSuccess) return e;
         if (dev >= 0 && dev < 64) configured[dev] = true;
     }
-    // the slices of the residuals and of W_int (the scale factors' matrices as one of scales * N rows)
+    // the slices of the residuals and of W_int (the scale factors' matrices as one of scales * rows rows)
     CUtensorMap xmap, wmap, imap;
-    const uint64_t rows = uint64_t(scales) * uint64_t(N);
-    if ((e = search_tensor_map(&wmap, resid, false, rows, uint64_t(K), uint32_t(kSearchRows), true)) != cudaSuccess) return e;
-    if ((e = search_tensor_map(&imap, offsets, true, rows, uint64_t(K), uint32_t(kSearchRows), false)) != cudaSuccess) return e;
-    const unsigned row_tiles = unsigned((N + kSearchRows - 1) / kSearchRows);
+    const uint64_t all = uint64_t(scales) * uint64_t(rows);
+    if ((e = search_tensor_map(&wmap, resid, false, all, uint64_t(K), uint32_t(kSearchRows), true)) != cudaSuccess) return e;
+    if ((e = search_tensor_map(&imap, offsets, true, all, uint64_t(K), uint32_t(kSearchRows), false)) != cudaSuccess) return e;
+    const unsigned row_tiles = unsigned((rows + kSearchRows - 1) / kSearchRows);
     // the error is a sum over tokens: pieces of at most 256 tokens, one launch each, the later ones adding to err_rows
-    // (pieces of about equal size, multiples of 16)
-    const int pieces = (T + kSearchMaxT - 1) / kSearchMaxT, piece = ((T + pieces - 1) / pieces + 15) / 16 * 16;
+    const int piece = search_piece(T);
     for (int t0 = 0; t0 < T; t0 += piece) {
         const int Tp = T - t0 < piece ? T - t0 : piece;
         p.X = reinterpret_cast<const __half *>(X) + size_t(t0) * K;
@@ -537,7 +562,12 @@ cudaError_t launch_search_errors(const uint16_t *resid, const uint8_t *offsets, 
         e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    search_sum_kernel<<<unsigned(P) * unsigned(scales), 256, 0, st>>>(err_rows, N, err);
+    return cudaSuccess;
+}
+
+cudaError_t launch_search_sums(const float *err_rows, int N, int candidates, double *err, cudaStream_t st)
+{
+    search_sum_kernel<<<unsigned(candidates), 256, 0, st>>>(err_rows, N, err);
     return cudaGetLastError();
 }
 

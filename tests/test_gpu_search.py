@@ -131,3 +131,35 @@ def test_grid_search_fullsize_sampled_rows(T):
 ])
 def test_grid_search_on_both_sides_of_its_rules(N, K, T, q, group, n_bits, n_scales):
     _check(N, K, T, q, group, n_bits, n_scales, f"search2/{N}x{K}x{T}")
+
+
+@pytest.mark.parametrize("N,K,T,group,n_scales,scratch", [(700, 512, 64, 128, 8, True), (392, 320, 80, 64, 9, False), (520, 256, 272, 0, 2, True),
+                                                          (72, 256, 32, 128, 1, False)])
+def test_grid_search_by_rows(N, K, T, group, n_scales, scratch):
+    """However many rows the workspace lets it search at a time: the same bits.  (A workspace for all rows; the one asked for; 72
+    rows with little more than a byte per weight: fewer rows than a block takes.)"""
+    import ctypes
+    n_bits, q = 4, 3
+    W, X = (torch.from_numpy(a).to(DEV) for a in _inputs(f"rows/{N}x{K}", N, K, T))
+    parts, s = bq.partitions(n_bits, q), bq.reexplore_factors(n_bits, n_scales)
+    d, P = bq.desc(N, K, q, group), len(parts)
+    asked = bq.lib().bcq_grid_search_workspace(ctypes.byref(d), T, n_bits, P, n_scales, 0 if scratch else 1)
+    G, t = (K // group if group else 1), min(n_scales, 8)
+    ample = asked + 4 * t * N * K
+    least = (t * N * K + (2 * t + q + 1) * (2 * N * G) + q * N * K // 8 + 512 * P + 8 * n_scales * P + 256 * 32 +
+             (4 * t * P * N if scratch else 0))
+    got = []
+    for size in (ample, asked, min(asked, least)):
+        ws = torch.zeros(size, dtype=torch.uint8, device=DEV)
+        err = torch.zeros((n_scales, P), dtype=torch.float64, device=DEV)
+        rows = None if scratch else torch.full((n_scales, P, N), float("nan"), dtype=torch.float32, device=DEV)
+        best = torch.full((2,), -1, dtype=torch.int32, device=DEV)
+        ptr = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+        assert bq.lib().bcq_grid_search(ctypes.byref(d), W.data_ptr(), X.data_ptr(), T, n_bits, ptr(parts), P, ptr(s), n_scales, err.data_ptr(),
+                                        None if scratch else rows.data_ptr(), best.data_ptr(), ws.data_ptr(), size, 0) == bq.OK
+        torch.cuda.synchronize()
+        got.append((err, best) if scratch else (err, best, rows))
+    assert bq.lib().bcq_poll_status() == bq.OK
+    for other in got[1:]:
+        assert all(torch.equal(a, b) for a, b in zip(got[0], other))
+    assert torch.isfinite(got[0][0]).all() and got[0][0].min() > 0

@@ -261,3 +261,14 @@ def test_stream_handle_without_torchs_private_functions(monkeypatch, missing):
     assert bq._stream() == 8
     monkeypatch.setattr(bq, missing, None)
     assert bq._stream() == 4242
+
+
+@pytest.mark.parametrize("N,K,q,group,P,scales", [(28672, 8192, 3, 128, 25, 8), (28672, 7168, 2, 64, 15, 8), (4096, 4096, 3, 128, 25, 8),
+                                                  (7168, 7168, 3, 0, 25, 3), (512, 1024, 2, 64, 7, 1)])
+def test_search_workspace_is_at_most_a_byte_per_weight_and_factor_or_a_gib(N, K, q, group, P, scales):
+    d = bq.desc(N, K, q, group)
+    need = bq.lib().bcq_grid_search_workspace(ctypes.byref(d), 128, 5, P, scales, 1)
+    G = K // group if group else 1
+    operand = q * N * K // 8 + (q + 1) * N * G * 2
+    small = P * (260 + 8 * scales) + 256 * 32
+    assert need <= max(scales * (N * K + 2 * N * G * 2) + operand, 2 ** 30) + small
