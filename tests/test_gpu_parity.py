@@ -467,17 +467,15 @@ def small_batch(N, K, q, group, rb, ks, codes, alpha, z, X):
     return Y.cpu().numpy()
 
 
-@pytest.mark.parametrize("N,W,q,ks,rb,B", [(40, 4, 3, 4, 2, 3), (16, 64, 1, 64, 1, 2), (24, 128, 2, 128, 2, 9), (16, 16, 4, 16, 1, 16)])
-def test_small_batch_splits_carry_any_partial_sum(N, W, q, ks, rb, B):
-    """Rows 0 .. 5: +inf and -inf in different splits; an infinity beside a large finite sum of the other sign; each alone; finite
-    sums of 3.8e9 that cancel to 30000; one of 32000 in a single split."""
-    K, group = 512 * W, 128
-    p, codes, alpha, z, X = make_layer(f"carry/{N}x{K}q{q}", N, K, q, group, B)
-    X = np.random.default_rng(W).integers(400, 600, X.shape).astype(np.float16)
+def far_apart_sums(N, K, q, B):
+    """Groups of 128; in rows 0 .. 5, at the two ends of K: +inf and -inf; an infinity and a large finite sum of the other sign;
+    each infinity alone; finite sums of 3.8e9 that cancel to 30000; one of 32000."""
+    p, codes, alpha, z, X = make_layer(f"carry/{N}x{K}q{q}", N, K, q, 128, B)
+    X = np.random.default_rng(K // 512).integers(400, 600, X.shape).astype(np.float16)
     X[:, -128:] = X[:, :128]
     X[:, -1] -= np.float16(0.5)                       # 60000 times the difference: 30000
     alpha, z = alpha.copy(), np.zeros_like(z)
-    alpha[:, :, :4], alpha[:, :, -4:] = 0, 0          # the first and the last window (different splits): offsets only
+    alpha[:, :, :4], alpha[:, :, -4:] = 0, 0          # the first and the last 512 weights: offsets only
     z[0, 0], z[0, -1] = np.inf, -np.inf
     z[1, 0], z[1, -1] = np.inf, -60000.0
     z[2, 0] = np.inf
@@ -485,14 +483,36 @@ def test_small_batch_splits_carry_any_partial_sum(N, W, q, ks, rb, B):
     z[4, 0], z[4, -1] = 60000.0, -60000.0
     z[5, 1] = 0.5
     with np.errstate(invalid="ignore"):
-        ref = oracle.forward_planes(p, alpha, z, X, group)
-    y = small_batch(N, K, q, group, rb, ks, codes, alpha, z, X).astype(np.float64)
+        return codes, alpha, z, X, oracle.forward_planes(p, alpha, z, X, 128)
+
+
+def check_far_apart_sums(y, ref, cancelled):
+    y = y.astype(np.float64)
     assert np.isnan(ref[:, 0]).all() and np.isnan(y[:, 0]).all()
     assert (y[:, 1] == np.inf).all() and (y[:, 2] == np.inf).all() and (y[:, 3] == -np.inf).all()
-    # row 4's sum is of the order of 3.8e9 until the last split is added: half an fp32 step, 2^7, per addition
-    assert np.abs(y[:, 4] - ref[:, 4]).max() <= 2.0 ** 7 * W
+    assert cancelled < 20000 and np.abs(y[:, 4] - ref[:, 4]).max() <= cancelled
     # fp32 sums, then one rounding to fp16
     assert np.abs(y[:, 5:] - ref[:, 5:]).max() <= 2.0 ** -10 * np.abs(ref[:, 5:]).max()
+
+
+@pytest.mark.parametrize("N,W,q,ks,rb,B", [(40, 4, 3, 4, 2, 3), (16, 64, 1, 64, 1, 2), (24, 128, 2, 128, 2, 9), (16, 16, 4, 16, 1, 16)])
+def test_small_batch_splits_carry_any_partial_sum(N, W, q, ks, rb, B):
+    """Infinities, and finite sums beyond what a split-K word holds, in different splits."""
+    codes, alpha, z, X, ref = far_apart_sums(N, 512 * W, q, B)
+    # row 4's sum may be of the order of 3.8e9 until the last split is added: half an fp32 step, 2^7, per addition
+    check_far_apart_sums(small_batch(N, 512 * W, q, 128, rb, ks, codes, alpha, z, X), ref, 2.0 ** 7 * W)
+
+
+@pytest.mark.parametrize("N,K,q,B", [(24, 4096, 3, 1), (16, 1152, 2, 16), (2500, 1024, 1, 2)])
+def test_canonical_products_carry_any_partial_sum(N, K, q, B):
+    """The same in the warps and the blocks of a cluster that share a row."""
+    codes, alpha, z, X, ref = far_apart_sums(N, K, q, B)
+    L = gpu_layer(N, K, q, 128, bq.LAYOUT_CANONICAL, codes, alpha, z)
+    Y = torch.zeros((B, N), dtype=torch.float16, device=DEV)
+    bq.gemm_smallbatch(L.d, L.packed, L.alpha, L.z, dev(X), Y, B, None)
+    torch.cuda.synchronize()
+    # two warps may carry row 4's 3.8e9 through all their K / 1024 + 1 segments' q + 1 additions each, then eight warps and blocks
+    check_far_apart_sums(Y.cpu().numpy(), ref, 2.0 ** 7 * (2 * (K / 1024 + 1) * (q + 1) + 16))
 
 
 @pytest.mark.parametrize("N,W,q,ks,rb,B", [(48, 16, 3, 16, 3, 2), (16, 64, 1, 64, 1, 11), (128, 8, 2, 4, 2, 8)])
