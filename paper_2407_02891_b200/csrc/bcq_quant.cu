@@ -137,16 +137,18 @@ __device__ __forceinline__ void warp_ranges(const __half *const (&w)[M], int L, 
     __half2 lo2[M], hi2[M];
 #pragma unroll
     for (int m = 0; m < M; ++m) lo2[m] = hi2[m] = __half2half2(w[m][0]);
-#pragma unroll (M == 1 ? 8 : 1)
-    for (int k = 8 * lane; k < L; k += 256) {   // L is a multiple of 32: whole 16-byte pieces
-        uint4 raw[M];
+    constexpr int kAtOnce = M == 1 ? 8 : 1;   // 16-byte pieces of a group on their way together (L is a multiple of 32)
+    for (int k = 8 * lane; k < L; k += 256 * kAtOnce) {
+        uint4 raw[M][kAtOnce];
 #pragma unroll
-        for (int m = 0; m < M; ++m) raw[m] = *reinterpret_cast<const uint4 *>(w[m] + k);
+        for (int m = 0; m < M; ++m)
+#pragma unroll
+            for (int c = 0; c < kAtOnce; ++c) raw[m][c] = *reinterpret_cast<const uint4 *>(w[m] + min(k + 256 * c, L - 8));   // (the last one again)
 #pragma unroll
         for (int m = 0; m < M; ++m) {
-            const __half2 *h = reinterpret_cast<const __half2 *>(&raw[m]);
+            const __half2 *h = reinterpret_cast<const __half2 *>(raw[m]);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) lo2[m] = __hmin2(lo2[m], h[i]), hi2[m] = __hmax2(hi2[m], h[i]);
+            for (int i = 0; i < 4 * kAtOnce; ++i) lo2[m] = __hmin2(lo2[m], h[i]), hi2[m] = __hmax2(hi2[m], h[i]);
         }
     }
     uint32_t both[M];   // (minimum, maximum) of a group, combined over the lanes
