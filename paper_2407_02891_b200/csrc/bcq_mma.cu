@@ -20,7 +20,7 @@
 //
 // Split K: as in the batch-1 kernel, every output owns one 64-bit word of the workspace, to which a split adds its
 // fixed-point sum and an arrival; whoever completes a word stores y and clears the word.  A sum that the word cannot hold
-// (infinite, not a number, very large) arrives as such, and whoever completes the word computes that output over all of K.
+// (infinite, not a number, very large) arrives as such, and the warp that completes the word computes that output over all of K.
 // The result does not depend on the order of arrival.  (fp32 sums per split, added up by the last to arrive, take a fence and
 // two more round trips to L2, and leave the adding to the last block: 8192 x 8192, 8 columns, 4 splits 21.6 us against 19.5;
 // 2048 x 8192, 16 splits 14.6 against 6.9.)  All waits are bounded.
@@ -38,7 +38,7 @@ constexpr int kMmaSmemBytes = 232448;    // 227 KB: the per-block opt-in maximum
 constexpr int kMmaFixedBytes = 1024;     // barriers and flags
 constexpr int kMmaMaxSlotsPerWarp = 4;
 
-static_assert(8 * kMmaWarps * kMmaMaxSlotsPerWarp + 8 <= kMmaFixedBytes, "barrier area");
+static_assert(8 * kMmaWarps * kMmaMaxSlotsPerWarp + 4 * (1 + kMmaWarps) <= kMmaFixedBytes, "barrier area");
 
 // Split-K words: arrivals in the top bits, below them the arrivals whose sum is not in the word, then the sum of the
 // biased fixed-point partial sums.  The widths follow from the number of arrivals.  The unit is 2^-36, so that
@@ -89,7 +89,6 @@ struct MmaParams {
     int N, K, B;
     int u_base, u_rem, w_base, w_rem;   // even partitions: part r starts at r * base + min(r, rem), base + (r < rem) items
     int split;               // k_splits > 1
-    View view;               // the operand, for outputs that are computed on their own
     int phase_windows;       // windows whose x is staged at a time
     int depth;               // ring slots per warp
     int x_at, sum_at, ring_at;   // shared memory: constants and x; sums between phases; rings
@@ -99,40 +98,112 @@ struct MmaParams {
 
 enum { kMmaWaitFull = 11, kMmaWaitDrain = 14 };
 
-// Outputs whose sum did not fit its split-K word, one after the other, by the whole warp: lane l has those of `which` (bit e:
-// row unit ua + (e / 2) % 2, column as in the kernel).  A lane takes every 32nd segment of 128 weights; signed sums of 128 in fp32 as in
-// the kernel, everything else in fp64.
-__device__ __noinline__ void mma_single_outputs(const MmaParams &p, int ua, unsigned which)
+struct MmaOnes {   // every non-zero is 1
+    uint32_t v[4];
+    __device__ const uint32_t (&operator()(int, int) const)[4] { return v; }
+};
+
+// Outputs whose sum did not fit their split-K words: one warp computes the pair of row units at ua (units from u1 on belong to
+// other blocks) over all of K, segment by segment as the kernel does, the segments in fp64, and stores this lane's outputs in
+// `which` (bit e: row unit ua + (e / 2) % 2, column as in the kernel).  The warp's ring, free by then, holds eight columns of a
+// segment of x.  Ends early once all of the outputs are NaN: a column of NaN costs 3 us at 8192 x 8192, 8 columns (1.8 ms with a
+// scalar product per output).
+template <int Q, bool GROUPED, bool WIDE>
+__device__ __forceinline__ void mma_whole_pair(const MmaParams &p, int ua, int u1, unsigned which)
 {
-    const int lane = threadIdx.x & 31;
-    for (int e = 0; e < 8; ++e) {
-        for (unsigned lanes = __ballot_sync(0xffffffffu, (which >> e) & 1u); lanes; lanes &= lanes - 1) {
-            const int from = __ffs(lanes) - 1;   // its row and column
-            const int n = (ua + ((e >> 1) & 1)) * kUnitRows + (from >> 2), b = 8 * (e >> 2) + 2 * (from & 3) + (e & 1);
-            const __half *x = p.X + size_t(b) * p.K;
-            double sum = 0.0;
-            for (int seg = lane; seg < p.K / 128; seg += 32) {
-                const int g = p.view.group ? seg : 0;
-                float total = 0.f, plane[4] = {0.f, 0.f, 0.f, 0.f};
-                for (int kb = 16 * seg; kb < 16 * seg + 16; ++kb) {
-                    uint32_t bits[4];
+    extern __shared__ __align__(128) unsigned char smem[];
+    constexpr int T = Q * 512 + (GROUPED ? Q * 64 + 64 : 0), HALVES = WIDE ? 2 : 1, NA = 4 * HALVES;
+    const int lane = threadIdx.x & 31, m = lane >> 2, t = lane & 3, U = p.N / kUnitRows;
+    const int next_unit = ua + 1 < u1 ? 1 : 0;   // (an odd block's last unit stands in for the one it does not have)
+    const int half_lo = m * 16 + 2 * ((2 * t - m) & 7), half_hi = m * 16 + 2 * ((2 * t + 1 - m) & 7);
+    unsigned char *buf = smem + p.ring_at + int(threadIdx.x >> 5) * p.depth * 2 * T;
+    const MmaOnes unit = {{p.ones, p.ones, p.ones, p.ones}};
+    double acc[NA];
 #pragma unroll
-                    for (int i = 0; i < 4; ++i) bits[i] = i < p.view.q ? *p.view.plane_byte(i, n, kb) : 0u;
-                    for (int j = 0; j < 8; ++j) {
-                        const float v = __half2float(x[8 * kb + j]);
-                        total += v;
+    for (int e = 0; e < NA; ++e) acc[e] = 0.0;
+    for (int seg = 0; seg < p.K / 128; ++seg) {
+        const unsigned char *tile = p.tiles + (size_t(seg >> 2) * U + ua) * T;
+        uint4 raw[HALVES][4];   // lane = (column of eight, word): 32 activations
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) plane[i] += (bits[i] >> j) & 1u ? v : -v;
-                    }
-                }
-                sum += double(__half2float(__ushort_as_half(*p.view.z_elem(n, g)))) * double(total);
+        for (int half = 0; half < HALVES; ++half) {
+            const int b = 8 * half + m;
+            const uint4 *src = reinterpret_cast<const uint4 *>(p.X + size_t(b) * p.K + 128 * size_t(seg) + 32 * t);
 #pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (i < p.view.q) sum += double(__half2float(__ushort_as_half(*p.view.alpha_elem(i, n, g)))) * double(plane[i]);
-            }
-            for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-            if (lane == 0) p.Y[size_t(b) * p.N + n] = __double2half(sum);
+            for (int j = 0; j < 4; ++j) raw[half][j] = b < p.B ? __ldg(src + j) : make_uint4(0u, 0u, 0u, 0u);
         }
+        uint32_t bits[Q][2];
+        __half scale[2][Q + 1];
+#pragma unroll
+        for (int i = 0; i < Q; ++i)
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const unsigned char *at = tile + i * 512 + 128 * (seg & 3) + (h ? half_hi : half_lo);
+                bits[i][h] = __byte_perm(__ldg(reinterpret_cast<const uint16_t *>(at)), __ldg(reinterpret_cast<const uint16_t *>(at + next_unit * T)), 0x5410u);
+            }
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int i = 0; i <= Q; ++i) {
+                const int u = ua + h * next_unit;
+                const uint16_t *at;
+                if constexpr (GROUPED)
+                    at = reinterpret_cast<const uint16_t *>(tile + h * next_unit * T + Q * 512) + (8 * (seg & 3) + m) * (Q + 1) + i;
+                else
+                    at = i < Q ? p.alpha + (size_t(u) * Q + i) * kUnitRows + m : p.z + size_t(u) * kUnitRows + m;
+                scale[h][i] = __ushort_as_half(__ldg(at));
+            }
+#pragma unroll
+        for (int half = 0; half < HALVES; ++half) {
+            __syncwarp();   // the staged columns have been read
+            float x = stage_word(raw[half], buf + m * kXSegBytes, t);
+            x += __shfl_xor_sync(0xffffffffu, x, 1);
+            x += __shfl_xor_sync(0xffffffffu, x, 2);
+            const float sums[2] = {__shfl_sync(0xffffffffu, x, 8 * t), __shfl_sync(0xffffffffu, x, 8 * t + 4)};   // of columns 2 t, 2 t + 1
+            __syncwarp();
+            float c[Q][4], none[1][4];
+            segment_sums<Q, false, true>(bits, buf + m * kXSegBytes + t * 16, buf, unit, c, none);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                double v = double(__half2float(scale[e >> 1][Q])) * double(sums[e & 1]);
+#pragma unroll
+                for (int i = 0; i < Q; ++i) v = fma(double(__half2float(scale[e >> 1][i])), double(c[i][e]), v);
+                acc[4 * half + e] += v;
+            }
+        }
+        bool open = false;
+#pragma unroll
+        for (int e = 0; e < NA; ++e) open = open || (((which >> e) & 1u) && acc[e] == acc[e]);
+        if (!__any_sync(0xffffffffu, open)) break;
+    }
+#pragma unroll
+    for (int e = 0; e < NA; ++e)
+        if ((which >> e) & 1u)
+            p.Y[size_t(8 * (e >> 2) + 2 * t + (e & 1)) * p.N + size_t(ua + ((e >> 1) & 1)) * kUnitRows + m] = __double2half(acc[e]);
+    __syncwarp();
+}
+
+// An output that is to be computed over all of K keeps the mark of the warp that completed its split-K word in it until the end
+// of the kernel, which has no registers to spare for a list, nor for what is found again here: the block's row units and
+// windows and the warp's pairs, as in the kernel.
+__device__ __forceinline__ unsigned mma_mark() { return blockIdx.y * kMmaWarps + (threadIdx.x >> 5) + 1; }
+template <int Q, bool GROUPED, bool WIDE>
+__device__ __noinline__ void mma_marked_outputs(const MmaParams &p)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, m = lane >> 2, t = lane & 3;
+    const int rbi = blockIdx.x, u0 = rbi * p.u_base + min(rbi, p.u_rem), u1 = u0 + p.u_base + (rbi < p.u_rem ? 1 : 0);
+    const int nwin = p.w_base + (int(blockIdx.y) < p.w_rem ? 1 : 0), P = (u1 - u0 + 1) >> 1;
+    const bool whole = nwin <= p.phase_windows;
+    const int run = (warp & 3) * (kMmaWarps / 4) + (warp >> 2), j0 = run * P * nwin / kMmaWarps, j1 = (run + 1) * P * nwin / kMmaWarps;
+    const int last = whole ? (j1 - 1) / nwin : P - 1;
+    for (int pair = whole ? j0 / nwin : warp; pair <= last; pair += whole ? 1 : kMmaWarps) {
+        const int ua = u0 + 2 * pair;
+        unsigned which = 0;
+        for (int e = 0; e < (WIDE ? 8 : 4); ++e) {
+            const int h = (e >> 1) & 1, b = 8 * (e >> 2) + 2 * t + (e & 1);
+            unsigned long long *word = p.accum + size_t(b) * p.N + size_t(ua + h) * kUnitRows + m;
+            if (ua + h < u1 && b < p.B && *word == mma_mark()) which |= 1u << e, *word = 0;
+        }
+        if (__any_sync(0xffffffffu, which != 0)) mma_whole_pair<Q, GROUPED, WIDE>(p, ua, u1, which);
     }
 }
 
@@ -205,6 +276,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) mma_gemm_kernel(const __grid_c
     if (lane == 0) {
         for (int s = 0; s < D; ++s) mbar_init(full0 + 8 * s, 1);
         if (tid == 0) *abort_flag = 0;
+        abort_flag[1 + warp] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         // weights are constants and may be fetched before the previous kernel in the stream has finished
@@ -215,11 +287,7 @@ __global__ void __launch_bounds__(kMmaThreads, 1) mma_gemm_kernel(const __grid_c
     asm volatile("griddepcontrol.wait;" ::: "memory");
 
     const int m = lane >> 2, t = lane & 3;
-    struct Ones {   // every non-zero is 1
-        uint32_t v[4];
-        __device__ const uint32_t (&operator()(int, int) const)[4] { return v; }
-    };
-    const Ones unit = {{p.ones, p.ones, p.ones, p.ones}};
+    const MmaOnes unit = {{p.ones, p.ones, p.ones, p.ones}};
     // chunk pairs 2 t and 2 t + 1 of row m's segment: the tile stores the segment's 16 chunks rotated by 2 m, so they sit
     // at half-words (2 t - m) mod 8 and (2 t + 1 - m) mod 8 of the row's 16 bytes
     const int half_lo = m * 16 + 2 * ((2 * t - m) & 7), half_hi = m * 16 + 2 * ((2 * t + 1 - m) & 7);
@@ -232,8 +300,6 @@ __global__ void __launch_bounds__(kMmaThreads, 1) mma_gemm_kernel(const __grid_c
     for (int e = 0; e < NA; ++e) acc[e] = 0.f;
 
     // outputs of one finished pair: rows m of both units, columns 2 t, 2 t + 1 (and 8 + those)
-    int emitted = 0, emitted0 = 0;       // this warp's pairs so far (at most 7), and the first of them
-    unsigned long long single = 0;       // 8 bits per pair: this lane's outputs that are to be computed on their own
     auto emit = [&](int pair) {
         const int ua = u0 + 2 * pair;
         unsigned long long before[NA], mine[NA];
@@ -252,21 +318,17 @@ __global__ void __launch_bounds__(kMmaThreads, 1) mma_gemm_kernel(const __grid_c
             }
         }
         if (p.split) {
-            unsigned which = 0;
 #pragma unroll
             for (int e = 0; e < NA; ++e) {
                 const int h = (e >> 1) & 1, b = 8 * (e >> 2) + 2 * t + (e & 1);
                 const size_t at = size_t(b) * p.N + size_t(ua + h) * kUnitRows + m;
                 if (ua + h < u1 && b < p.B && split_complete(before[e], p.fmt)) {
-                    if (split_odd(before[e] + mine[e], p.fmt))
-                        which |= 1u << e;
-                    else
-                        p.Y[at] = split_decode(before[e] + mine[e], p.fmt);
-                    p.accum[at] = 0;
+                    const bool odd = split_odd(before[e] + mine[e], p.fmt);
+                    if (!odd) p.Y[at] = split_decode(before[e] + mine[e], p.fmt);
+                    p.accum[at] = odd ? mma_mark() : 0;
+                    if (odd) abort_flag[1 + warp] = 1;   // some of the warp's outputs carry its mark
                 }
             }
-            single |= (unsigned long long)which << (8 * emitted);
-            if (emitted++ == 0) emitted0 = pair;
         }
     };
 
@@ -449,9 +511,8 @@ __global__ void __launch_bounds__(kMmaThreads, 1) mma_gemm_kernel(const __grid_c
         }
     }
 
-    if (__any_sync(0xffffffffu, single != 0))
-        for (int i = 0; i < emitted; ++i)
-            mma_single_outputs(p, u0 + 2 * (emitted0 + i * (whole ? 1 : kMmaWarps)), unsigned(single >> (8 * i)) & 0xffu);
+    __syncwarp();
+    if (alive && abort_flag[1 + warp]) mma_marked_outputs<Q, GROUPED, WIDE>(p);   // (the warp's ring is free now)
 
     // Gave up on a wait: copies this warp started may still be in flight.  See them land (bounded)
     // before the block's shared memory can be handed to another block.
@@ -555,10 +616,9 @@ cudaError_t launch_mma_gemm(const bcq_desc &d, const bcq_plan &plan, const void 
     prm.ones = 0x3C003C00u;
     prm.split = splits > 1;
     prm.fmt = split_format(splits);
-    prm.view = make_view(d, packed, alpha, z);
     const bool grouped = d.group != 0;
     const int windows = prm.w_base + (prm.w_rem ? 1 : 0), pairs = (prm.u_base + (prm.u_rem ? 1 : 0) + 1) / 2;
-    const MmaLayout l = mma_layout(d.q, grouped, B, windows, pairs);
+    const MmaLayout l = mma_layout(d.q, grouped, B, windows, pairs);   // (a warp's ring is at least 2 KB: mma_whole_pair)
     if (l.phase_windows < 1 || l.depth < 1) return cudaErrorInvalidValue;
     prm.phase_windows = l.phase_windows, prm.depth = l.depth;
     prm.x_at = l.x_at, prm.sum_at = l.sum_at, prm.ring_at = l.ring_at;

@@ -515,6 +515,28 @@ def test_canonical_products_carry_any_partial_sum(N, K, q, B):
     check_far_apart_sums(Y.cpu().numpy(), ref, 2.0 ** 7 * (2 * (K / 1024 + 1) * (q + 1) + 16))
 
 
+@pytest.mark.parametrize("N,K,q,group,rb,ks,B", [(40, 2048, 3, 128, 2, 4, 5), (72, 1536, 1, 0, 1, 3, 16), (24, 1024, 4, 0, 1, 2, 3), (1400, 8704, 2, 128, 1, 2, 12)])
+def test_small_batch_columns_that_are_not_numbers(N, K, q, group, rb, ks, B):
+    """A column of NaN, a column with one infinity, activations of 65504 (sums beyond the split-K words, most of them beyond fp16):
+    the other columns' bits are not disturbed, and these come out as the oracle has them."""
+    p, codes, alpha, z, X = make_layer(f"nan/{N}x{K}q{q}", N, K, q, group, B)
+    clean = small_batch(N, K, q, group, rb, ks, codes, alpha, z, X)
+    X = X.copy()
+    X[0], X[1, K // 2] = np.nan, np.inf
+    X[2] = np.copysign(np.float16(65504.0), X[2])
+    with np.errstate(invalid="ignore", over="ignore"):
+        ref = oracle.forward_planes(p, alpha, z, X, group)
+        want = ref.astype(np.float16).astype(np.float64)
+    y = small_batch(N, K, q, group, rb, ks, codes, alpha, z, X)
+    assert np.array_equal(y[3:].view(np.uint16), clean[3:].view(np.uint16))
+    assert np.isnan(y[0]).all()
+    assert np.array_equal(np.isnan(y[1]), np.isnan(want[1])) and np.array_equal(y[1][~np.isnan(want[1])], want[1][~np.isnan(want[1])])
+    y2, near = y[2].astype(np.float64), np.abs(np.abs(ref[2]) - 65520.0) < 64.0   # (next to the largest fp16 number either side is right)
+    assert np.array_equal(np.isinf(y2[~near]), np.isinf(want[2][~near])) and np.isinf(want[2]).any()
+    finite = np.isfinite(y2) & ~near
+    assert finite.any() and np.abs(y2 - ref[2])[finite].max() <= 2.0 ** 6
+
+
 @pytest.mark.parametrize("N,W,q,ks,rb,B", [(48, 16, 3, 16, 3, 2), (16, 64, 1, 64, 1, 11), (128, 8, 2, 4, 2, 8)])
 def test_small_batch_splits_keep_small_sums(N, W, q, ks, rb, B):
     """Outputs around 2^-16, below fp16's normal range: the one rounding to a multiple of 2^-24 is all that may be lost.  The
