@@ -16,8 +16,8 @@
 // one scale per row) take the range first, eight rows per block, and read the rows a second time from L2.
 //
 // Bound: instruction issue, then HBM (2 bytes per weight).  7168 x 7168, q = 3, groups of 128: 201 us with a chunk of 8 weights per
-// thread, byte stores and a 16-lane range reduction; 52.9 us with 32 weights per lane; 49.8 us (2.6 TB/s) without the comparison
-// with the top integer where no weight lies beyond it, and with integers of up to 4 bits looked up two at a time.
+// thread, byte stores and a 16-lane range reduction; 52.9 us with 32 weights per lane; 49.5 us with integers of up to 4 bits looked up
+// two at a time; 47.1 us (2.7 TB/s) without the comparison with the top integer where no weight lies beyond it.
 #include "bcq_planes.cuh"
 
 namespace bcq {
@@ -79,6 +79,9 @@ struct IntDecision {
         if (!plain) inv = 0.f;
         ceiling = __float_as_int(kBase + float(top) + 0.5f);
     }
+    // Whether the integer part for this weight is above the top: half a unit above the ceiling, which is the middle of the top
+    // integer's cell (fractions up to there are one half and more, and never in doubt).  NaN counts as above.
+    __device__ bool beyond_top(float w) const { return __float_as_int(fmaf(w, inv, c)) >= ceiling + (1 << (FR - 1)); }
 };
 
 // Integers of the 8 weights of one 16-byte piece, one per byte.  CLAMP: some weight may lie beyond the top integer.
@@ -327,9 +330,9 @@ __global__ void __launch_bounds__(256, 3) rtn_kernel(const __half *__restrict__ 
         }
         const IntDecision<FR> dec(s_h, b_h, lo, hi, tab.top);
         uint2 ints[4];
-        // The quotient grows with the weight: where the largest weight's is not beyond the top integer, none is (always so with
-        // scale factors of 1 and more, but for scales among the smallest numbers).
-        if (__any_sync(0xffffffffu, __float_as_int(fmaf(hi, dec.inv, dec.c)) > dec.ceiling)) {
+        // The quotient grows with the weight: where the largest weight's rounds to the top integer or less, every weight's does
+        // (with scale factors of 1 and more that is every group but those whose scale is among the smallest numbers).
+        if (__any_sync(0xffffffffu, dec.beyond_top(hi))) {
 #pragma unroll
             for (int c = 0; c < 4; ++c) ints[c] = piece_ints<FR, true>(raw[c], dec, s_h, b_h, tab.top);
         } else {

@@ -229,8 +229,8 @@ def test_quantize_rtn_in_parts(N, K, q, group):
 @pytest.mark.parametrize("N,K,group,layout,s_factor", [
     (24, 1024, 128, bq.LAYOUT_TILED, 1.0), (24, 1024, 64, bq.LAYOUT_TILED, 0.6), (17, 1184, 32, bq.LAYOUT_CANONICAL, 1.0), (9, 1152, 0, bq.LAYOUT_CANONICAL, 0.9)])
 def test_quantize_rtn_clamps_where_a_weight_lies_beyond_the_top(N, K, group, layout, s_factor, n_bits):
-    """Ordinary groups next to groups whose scale is a subnormal number, rounded down by up to a half: only in those (or with a
-    factor below one) does a quotient lie beyond the top integer.  Integers of up to four bits are looked up in pairs."""
+    """Blocks of 32 subnormal weights strewn among ordinary ones, factors of one and below: a quotient beyond the top integer in some
+    groups of 32 at 3 and 4 bits and, with the factors below one, in every group.  Integers of up to four bits are looked up in pairs."""
     rng = np.random.default_rng(N + K + n_bits)
     W = weights(f"top/{N}x{K}", N, K)
     small = rng.random((N, K // 32)) < 0.3
@@ -242,3 +242,54 @@ def test_quantize_rtn_clamps_where_a_weight_lies_beyond_the_top(N, K, group, lay
     assert same(S, e_S) and same(qb, e_qb) and same(wi, e_wi) and same(packed, e_packed)
     if a is not None:
         assert same(a, e_a) and same(z, e_z)
+
+
+def top_sides(W, S, qb, L, n_bits, lane_wise):
+    """(segments of eight rows that hold an integer beyond the top, segments whose largest quotients are below top + 0.4), by the
+    definition; the largest of 32 neighbouring weights where lane_wise, of a group otherwise."""
+    N, K = W.shape
+    G, top = K // L, 2 ** n_bits - 1
+    s = np.repeat(S.astype(np.float64).reshape(N, G), L, axis=1)
+    t = (W.astype(np.float64) - np.repeat(qb.astype(np.float64).reshape(N, G), L, axis=1)) / np.where(s > 0, s, np.inf)
+    run_len = 32 if lane_wise else L
+    largest = np.repeat(t.reshape(N, K // run_len, run_len).max(axis=2), run_len, axis=1)
+    beyond = within = 0
+    for n in range(0, N, 8):
+        for k in range(0, K, 128):
+            beyond += bool((np.rint(t[n:n + 8, k:k + 128]) > top).any())
+            within += bool((largest[n:n + 8, k:k + 128] < top + 0.4).all())
+    return beyond, within
+
+
+@pytest.mark.parametrize("n_bits", [2, 4, 5, 7, 8])
+@pytest.mark.parametrize("N,K,group,layout", [
+    (24, 1024, 128, bq.LAYOUT_TILED), (24, 1024, 64, bq.LAYOUT_TILED), (17, 1184, 32, bq.LAYOUT_CANONICAL), (12, 1152, 0, bq.LAYOUT_CANONICAL),
+    (24, 1536, 192, bq.LAYOUT_CANONICAL)])
+@pytest.mark.parametrize("factor", ["one", "line", "low"])
+def test_quantize_rtn_segments_with_and_without_integers_beyond_the_top(N, K, group, layout, n_bits, factor):
+    """A segment in which no quotient rounds to more than the top integer goes without the comparison with it.  Every second row
+    unit holds groups whose range is about 1.45 top of the smallest subnormal number, which is their scale: with a factor of one
+    their largest quotients, and no other group's, lie beyond the top.  With a factor just above top / (top + 1/2) the largest quotients
+    of ordinary groups lie about where the top integer's cell ends, well below it far beyond."""
+    rng = np.random.default_rng(1000 * n_bits + K + group)
+    L, top = group or K, 2 ** n_bits - 1
+    W = weights(f"sides/{N}x{K}/{n_bits}", N, K)
+    reach = top + max(1, 4 * top // 9)        # less than 1.5 top: the scale is rounded down to 2^-24
+    for n in range(8, N, 16):
+        for r in range(n, min(n + 8, N)):
+            for g in range(K // L):
+                if rng.random() < 0.3 or (r == n and g % 2 == 0):
+                    steps = rng.integers(0, reach + 1, L)
+                    steps[rng.permutation(L)[:2]] = 0, reach
+                    W[r, g * L:(g + 1) * L] = ((steps - 3) * 2.0 ** -24).astype(np.float16)
+    s_factor = {"one": 1.0, "line": 1.0005 * top / (top + 0.5), "low": 0.6}[factor]
+    q = min(n_bits, 3)
+    b2p = [i % q for i in range(n_bits)]
+    e_wi, e_S, e_qb, e_packed, e_a, e_z, _ = expected(W, q, group, layout, n_bits, b2p, s_factor)
+    beyond, within = top_sides(W, e_S, e_qb, L, n_bits, L not in (128, 64, 32))
+    assert beyond > 0 and (factor != "one" or within > 0)
+    for want_int in (True, False):
+        S, qb, wi, packed, a, z = run(W, q, group, layout, n_bits, b2p, s_factor, want_int)
+        assert same(S, e_S) and same(qb, e_qb) and same(packed, e_packed) and (wi is None or same(wi, e_wi))
+        if a is not None:
+            assert same(a, e_a) and same(z, e_z)
