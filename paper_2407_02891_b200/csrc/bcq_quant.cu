@@ -255,8 +255,9 @@ __device__ __forceinline__ void lanes_range(const uint4 (&raw)[NR], float &lo, f
 // LANES: lanes per group, 4, 2 or 1 for groups of 128, 64 and 32 (one pass; jobs = (row unit, segment), segments
 // fastest); 0 for any other group length L: a block takes the row unit blockIdx.x, ranges first, and of its segments the
 // part blockIdx.y (groups that two parts share are done by both, with the same results).
-// PAIRS: integers of at most 4 bits, looked up two at a time.
-template <int FR, int LANES, bool PAIRS>
+// PAIRS: integers of at most 4 bits, looked up two at a time.  VOTE: a warp asks whether any of its weights lies beyond the top
+// integer, and leaves the comparison out where none does; otherwise it compares them all.
+template <int FR, int LANES, bool PAIRS, bool VOTE>
 __global__ void __launch_bounds__(256, 3) rtn_kernel(const __half *__restrict__ W, const __grid_constant__ QuantTable tab, int L,
                                                   __half *S, __half *qbias, uint8_t *__restrict__ w_int, const View dst)
 {
@@ -332,7 +333,7 @@ __global__ void __launch_bounds__(256, 3) rtn_kernel(const __half *__restrict__ 
         uint2 ints[4];
         // The quotient grows with the weight: where the largest weight's rounds to the top integer or less, every weight's does
         // (with scale factors of 1 and more that is every group but those whose scale is among the smallest numbers).
-        if (__any_sync(0xffffffffu, dec.beyond_top(hi))) {
+        if (!VOTE || __any_sync(0xffffffffu, dec.beyond_top(hi))) {
 #pragma unroll
             for (int c = 0; c < 4; ++c) ints[c] = piece_ints<FR, true>(raw[c], dec, s_h, b_h, tab.top);
         } else {
@@ -392,15 +393,48 @@ static cudaError_t walk_grid(int N, int K, int per_sm, dim3 &grid)
     return cudaSuccess;
 }
 
+// Whether warps vote (VOTE above).  With factors above top / (top + 1/2) the largest weight of a group rounds to the top integer, but
+// for scales among the smallest numbers, and the comparison is left out nearly everywhere; with smaller factors every group has
+// weights beyond the top, and the vote is for nothing.  7168 x 7168, q = 3, tiled, with / without the vote, us:
+//   factor 1    groups of 128: 4 bits 44.5 / 47.2, 8 bits 52.3 / 54.2; of 64: 5 bits 49.8 / 51.5; of 32: 5 bits 48.1 / 49.7,
+//               8 bits 53.0 / 53.3 (canonical 56.0 / 55.8, of 1024 x 4096 9.53 / 9.43)
+//   factor 0.9  groups of 64: 5 bits 52.5 / 51.4, 8 bits 57.6 / 56.5; of 32: 5 bits 51.6 / 50.4, 8 bits 55.6 / 53.9; of 128: 8 bits
+//               55.1 / 54.5, but 5 bits 50.2 / 50.7; one scale per row: 8 bits 69.1 / 68.8, but 4 bits 59.8 / 60.7, 5 bits 60.7 / 61.4
+static bool rtn_votes(int n_bits, int lanes, double s_factor, double top)
+{
+    const bool inside = s_factor * (top + 0.5) > top;
+    if (n_bits == 8) return inside && lanes != 1;
+    return inside || lanes == 4 || lanes == 0;
+}
+
 template <int FR, bool PAIRS>
-static cudaError_t launch_rtn(const __half *w, const QuantTable &tab, __half *s, __half *b, uint8_t *w_int, const View &dst, cudaStream_t st)
+static auto rtn_kernel_of(int lanes, bool votes)
+{
+    if (lanes == 4) {
+        if constexpr (FR == 15)
+            if (!votes) return rtn_kernel<FR, 4, PAIRS, false>;
+        return rtn_kernel<FR, 4, PAIRS, true>;
+    }
+    if (lanes == 2) return votes ? rtn_kernel<FR, 2, PAIRS, true> : rtn_kernel<FR, 2, PAIRS, false>;
+    if (lanes == 1) {
+        if constexpr (FR != 15)
+            if (votes) return rtn_kernel<FR, 1, PAIRS, true>;
+        return rtn_kernel<FR, 1, PAIRS, false>;
+    }
+    if constexpr (FR == 15)
+        if (!votes) return rtn_kernel<FR, 0, PAIRS, false>;
+    return rtn_kernel<FR, 0, PAIRS, true>;
+}
+
+template <int FR, bool PAIRS>
+static cudaError_t launch_rtn(const __half *w, const QuantTable &tab, int n_bits, __half *s, __half *b, uint8_t *w_int, const View &dst, cudaStream_t st)
 {
     const int L = dst.group == 0 ? dst.K : dst.group;
     const int lanes = (L == 128 || L == 64 || L == 32) ? L / 32 : 0;
     dim3 grid;
     const cudaError_t e = lanes ? walk_grid(dst.N, dst.K, 3, grid) : unit_grid(dst.N, dst.K, 3, grid);
     if (e != cudaSuccess) return e;
-    const auto kernel = lanes == 4 ? rtn_kernel<FR, 4, PAIRS> : lanes == 2 ? rtn_kernel<FR, 2, PAIRS> : lanes == 1 ? rtn_kernel<FR, 1, PAIRS> : rtn_kernel<FR, 0, PAIRS>;
+    const auto kernel = rtn_kernel_of<FR, PAIRS>(lanes, rtn_votes(n_bits, lanes, tab.s_factor, tab.top));
     kernel<<<grid, 256, 0, st>>>(w, tab, L, s, b, w_int, dst);
     return cudaGetLastError();
 }
@@ -418,8 +452,8 @@ cudaError_t launch_quantize_rtn(const uint16_t *W, int n_bits, double s_factor, 
     const __half *w = reinterpret_cast<const __half *>(W);
     __half *s = reinterpret_cast<__half *>(S), *b = reinterpret_cast<__half *>(qbias);
     // 16 fraction bits leave 7 integer bits in the mantissa
-    if (n_bits <= 4) return launch_rtn<16, true>(w, tab, s, b, w_int, dst, st);
-    return n_bits <= 7 ? launch_rtn<16, false>(w, tab, s, b, w_int, dst, st) : launch_rtn<15, false>(w, tab, s, b, w_int, dst, st);
+    if (n_bits <= 4) return launch_rtn<16, true>(w, tab, n_bits, s, b, w_int, dst, st);
+    return n_bits <= 7 ? launch_rtn<16, false>(w, tab, n_bits, s, b, w_int, dst, st) : launch_rtn<15, false>(w, tab, n_bits, s, b, w_int, dst, st);
 }
 
 // ---- step 1 for the search: several scale factors in one pass over W -----------------------------------------------
