@@ -16,7 +16,8 @@ struct MergeTable {
 // codes[t] = code of w_int[t], 16 per thread and step (one 16-byte load and store; the 256-byte table sits in shared
 // memory, conflict-free up to 7 step-1 bits), and, by the blocks from code_blocks on, the fused scales:
 // alpha_j = S * m_j and z = S * centre + qbias, each evaluated exactly in fp64 (the products and the sum of two
-// fp16-derived values fit 53 bits) and rounded once to fp16.  Bound by HBM: one byte in, one byte out per weight.
+// fp16-derived values fit 53 bits) and rounded once to fp16.  Bound by the look-ups (load and store pipe 69 % busy at
+// 7168 x 7168, 19.6 us) beside HBM (38 %): one byte in, one byte out per weight.
 __global__ void __launch_bounds__(256) merge_kernel(const uint4 *__restrict__ w_int, uint4 *__restrict__ codes, size_t pieces, int code_blocks,
                                                     const __half *__restrict__ S, const __half *__restrict__ qbias, size_t units, int q,
                                                     __half *__restrict__ alpha, __half *__restrict__ z, const __grid_constant__ MergeTable tab)
@@ -73,9 +74,9 @@ cudaError_t launch_merge(const bcq_desc &d, const uint8_t *w_int, const uint16_t
 // eight of them fit one word (two nibbles per byte); plane i of the eight is one shift, one AND and one multiplication
 // that gathers the eight bits into the top byte (the products of the other bits fall below it or out of the word, and
 // no two of them meet).  A block walks many jobs, the next job's codes on their way while one is packed: a block's
-// closing fence costs more than a job.  Bound by HBM (codes mostly come from L2, right behind the merge) and, within a
-// factor of two, by instruction issue.  Merge and pack of 7168 x 7168, q = 3, groups of 128: 212 us as one byte per
-// thread and store, in four launches; 45 us so.
+// closing fence costs more than a job.  Bound by instruction issue (slots 63 % busy, 264 instructions per job) and the
+// latency of the codes (a third of a warp's time), HBM 31 % busy (codes not in L2).  Merge and pack of 7168 x 7168, q = 3,
+// groups of 128: 212 us as one byte per thread and store, in four launches; 44 us so.
 
 __device__ __forceinline__ uint32_t plane_word(const uint32_t (&z)[4], int i)
 {

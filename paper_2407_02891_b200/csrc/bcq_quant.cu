@@ -15,7 +15,7 @@
 // Groups of 128, 64 and 32 are 4, 2 and 1 of those lanes: range by shuffles, one pass over W.  Other group lengths (and
 // one scale per row) take the range first, eight rows per block, and read the rows a second time from L2.
 //
-// Bound: instruction issue, then HBM (2 bytes per weight).  7168 x 7168, q = 3, groups of 128: 201 us with a chunk of 8 weights per
+// Bound: instruction issue (slots 68 % busy, 20.6 instructions per weight), then HBM (2 bytes per weight).  7168 x 7168, q = 3, groups of 128: 201 us with a chunk of 8 weights per
 // thread, byte stores and a 16-lane range reduction; 52.9 us with 32 weights per lane; 49.5 us with integers of up to 4 bits looked up
 // two at a time; 47.1 us (2.7 TB/s) without the comparison with the top integer where no weight lies beyond it.
 #include "bcq_planes.cuh"
